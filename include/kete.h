@@ -246,13 +246,10 @@ int kete_propagate(kete_ctx *ctx, double *states, double *epochs, int64_t n, dou
 
 /* kete_propagate through a chain of stops every leg_days days (the survey's
  * batch-midpoint chain, Sec. 2, applied to a single target): the stops are
- * epochs[0] + k leg_days toward t_target (which ends the chain), so that
- * the bodies stay together in time and a step spanning a whole leg reads the
- * planets from rows shared by all bodies instead of evaluating the table.
- * The price is more steps wherever the natural step exceeds leg_days (with
- * 8-day legs, main-belt bodies and comet clones take about twice as many
- * steps, which outweighed the cheaper evaluations on GB300: 1.2-1.3x slower
- * than kete_propagate).  Results agree
+ * epochs[0] + k leg_days toward t_target (which ends the chain), no step
+ * passes one, and a step spanning a whole leg reads the planets from rows
+ * shared by all bodies.  kete_propagate shares rows for steps of any length
+ * and is the faster call; this one bounds the step.  Results agree
  * with a chain of stops on the same grid (kete_propagate_stops), not
  * bit for bit with kete_propagate (another step sequence; the difference is
  * at the integrator's truncation level).  Bodies at other epochs than
@@ -266,7 +263,9 @@ int kete_propagate_legs(kete_ctx *ctx, double *states, double *epochs, int64_t n
 /* Propagate n bodies (not modified) along the chain epoch -> stops[0] ->
  * stops[1] -> ... (host, [n_stops], ascending), carrying the step size along
  * the chain: the schedule kete_fov_check uses for the batch midpoints (Sec. 2,
- * "between the median observation times of consecutive batches").
+ * "between the median observation times of consecutive batches").  A step may
+ * pass stops: the states there are those of the step's collocation
+ * polynomial, whose error stays below the rounding of the positions.
  * out (device, [n_stops][6][n]) receives the states; a failed body gets NaN
  * from its failing stop on.  Errors: BAD_ARG, NO_EPHEM, CUDA. */
 int kete_propagate_stops(kete_ctx *ctx, const double *states, const double *epochs, int64_t n,
@@ -358,15 +357,17 @@ int kete_get_stats(const kete_ctx *ctx, kete_stats *out);
  * is launched by later calls: kind KETE_PROP_STATIC or
  * KETE_PROP_WORK_STEALING, block 32..128 threads (multiple of 32).  Both
  * produce identical results; they differ in load balance when bodies need
- * very different numbers of steps.  split_lanes 4, 8 or 16 (0 or 1: off) with
- * defer_steps > 0 adds a second phase: a body that has made more than
- * defer_steps step attempts per stop reached is set aside at a step boundary
- * and finished by a persistent launch in which split_lanes lanes share each
- * body's force evaluations (the masses split over the lanes, partial sums
- * combined by shuffles).  Which bodies are set aside depends on each body
+ * very different numbers of steps.  Long bodies are set aside at a step
+ * boundary and finished by a second launch with one warp per body: past a
+ * budget of attempts taken from the span or, with split_lanes 4, 8 or 16 (0 or
+ * 1: the automatic budget) and defer_steps > 0, past defer_steps attempts per
+ * stop reached (the three values of split_lanes act alike).  Without an
+ * explicit budget a call of few bodies takes one warp per body throughout; in
+ * that form every term is FP64 in both precisions.
+ * Which bodies are set aside depends on each body
  * alone, so the static and work-stealing schedules still agree bit for bit;
- * a set-aside body's force sums are added in another order than in one lane
- * (differences at the rounding level).  cost_order != 0: lanes take the bodies
+ * the two forms differ in the order of their sums and corrector sweeps
+ * (differences at the truncation level, ~1e-13 AU over a year).  cost_order != 0: lanes take the bodies
  * most expensive first (cost estimated from each body's heliocentric conic:
  * steps ~ integral dt / r^1.5), so a warp holds bodies of similar cost; this
  * changes only the schedule, not any result.  Default: work stealing, 128, no
@@ -377,8 +378,7 @@ int kete_set_propagation(kete_ctx *ctx, int precision, int kind, int block, int 
 
 /* Autotuner: time every launch variant (static 128, work stealing 64 and 128,
  * each in index and in cost order; work stealing 128 in cost order with long
- * bodies set aside after 64 attempts per stop for 8 or 4 lanes each, or after
- * 24 for 8 lanes) on an evenly spread sample of min(max_sample, n) of the n
+ * bodies set aside after 64 or 24 attempts per stop) on an evenly spread sample of min(max_sample, n) of the n
  * bodies (device states [6][n] / epochs [n], not modified), run on persistent
  * grids scaled down by sample / n so that each lane works through as many
  * bodies as in the whole run, propagated along

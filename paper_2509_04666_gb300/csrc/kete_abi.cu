@@ -27,8 +27,8 @@ enum Slot {
     S_EXPFIRST, S_XEPOCH, S_XOBS, S_XCEN, S_XCENF, S_XRAD, S_XCS, S_XBATCH, S_NEXT, S_BFIRST, S_BTREF,
     S_BO, S_BROBS, S_BTSPAN, S_BRMAX, S_BSUN, S_NBATCH, S_BANDS, S_CELLKEY, S_CELLCNT,
     S_CELLSTART, S_CELLCUR, S_CELLEXP, S_CAND, S_EXPCNT, S_EXPOFF, S_EXPCUR, S_CANDBODY,
-    S_HITTMP, S_FRAMECNT, S_FRAMEOFF, S_FRAMECUR, S_HITGROUP, S_MAXRAD, S_NT_T0, S_NT_H,
-    S_NT_R64, S_NT_R32, S_XSUN, S_XOBSREL, S_NEXTBODY, S_TUNE_ST, S_TUNE_EP, S_TUNE_OUT,
+    S_HITTMP, S_FRAMECNT, S_FRAMEOFF, S_FRAMECUR, S_HITGROUP, S_MAXRAD, S_GRID, S_GRID_OK,
+    S_GRID_R64, S_GRID_R32, S_STOPROW, S_XSUN, S_XOBSREL, S_NEXTBODY, S_TUNE_ST, S_TUNE_EP, S_TUNE_OUT,
     S_ADJ_REC, S_ADJ_NREC, S_ADJ_NBAT, S_ADJ_BIDX, S_ADJ_YREF, S_ADJ_GJUMP, S_ADJ_STATUS,
     S_KSTOP, S_DEFER_LIST, S_DEFER_CNT, S_ORDER, S_ORDER_KEY, S_ORDER_HIST, S_ORDER_OFF,
     S_ORDER_SCAN, S_ORDER_N, S_ADJ_TEND, S_LEG_OUT,
@@ -276,6 +276,7 @@ int kete_create(kete_ctx **out, int device, void *cuda_stream)
     std::memset(ctx->h_ctr, 0, sizeof(DevCounters));
     upload_radau_tables(ctx->stream);
     e = upload_adjoint_tables(ctx->stream);
+    if (e == cudaSuccess) e = upload_warp_tables(ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) {
         kete_destroy(ctx);
@@ -418,6 +419,7 @@ static int make_force(kete_ctx *ctx, const kete_force_model *fm_in, ForceDev &F)
         for (int c = 0; c < 3; c++) F.pole_m2_32[m][c] = (float)F.pole_m2[m][c];
     }
     F.eps = fm.eps;
+    F.log2_eps = (float)std::log2(fm.eps);
     F.eps_pc = fm.eps_pc;
     F.safety = fm.safety;
     F.dt_init = fm.dt_init;
@@ -442,12 +444,10 @@ extern "C" int kete_ephem_eval(kete_ctx *ctx, const double *t, int64_t n, int bo
 }
 
 // Bodies (states [6][stride] SoA, epochs [n], device) most expensive first
-// over [epoch, end]: end = the last stop (stops_dev, device) or t_end_i[i]
-// (device) per body.  *order_n receives a device copy of n, the kernels'
+// over [epoch, end]: end = t_end, or t_end_i[i] (device) per body.  *order_n receives a device copy of n, the kernels'
 // queue length.
 static int cost_order(kete_ctx *ctx, const double *states, int64_t stride, const double *epochs,
-                      int64_t n, const double *stops_dev, int n_stops, const double *t_end_i,
-                      const kete_nongrav *ng, int32_t **order, unsigned long long **order_n)
+                      int64_t n, double t_end, const double *t_end_i, const kete_nongrav *ng, int32_t **order, unsigned long long **order_n)
 {
     OrderScratch s;
     const size_t nh = order_hist_elems(n);
@@ -457,12 +457,6 @@ static int cost_order(kete_ctx *ctx, const double *states, int64_t stride, const
     GET(S_ORDER_OFF, nh + 1, s.off);
     GET(S_ORDER_SCAN, scan_tmp_elems((int64_t)nh), s.scan_tmp);
     GET(S_ORDER_N, 1, *order_n);
-    double t_end = 0.0;
-    if (!t_end_i) {
-        CUDA_TRY(cudaMemcpyAsync(&t_end, stops_dev + (n_stops - 1), sizeof(double),
-                                 cudaMemcpyDeviceToHost, ctx->stream));
-        CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-    }
     const unsigned long long nn = (unsigned long long)n;
     CUDA_TRY(cudaMemcpyAsync(*order_n, &nn, sizeof(nn), cudaMemcpyHostToDevice, ctx->stream));
     CUDA_TRY(order_by_cost(ctx->E, states, stride, epochs, n, t_end, t_end_i, ng, s, *order,
@@ -471,61 +465,196 @@ static int cost_order(kete_ctx *ctx, const double *states, int64_t stride, const
     return KETE_OK;
 }
 
-// Launch the propagation kernel with the context's variant for F's precision.
-// out_aos: stop k of body i at out[(k stride + i) * 6 + c] (see k_propagate)
-static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const double *stops_dev,
-                     int n_stops, double *out, int64_t stride, bool keep_on_fail,
-                     const NodeTable *nt, int leg0, bool out_aos = false)
+// Whether a call takes one warp per body throughout.  Measured in FP64: a step
+// takes a lane 0.45 ms and the full lane grid 0.025 us, a warp 0.03 ms and the
+// full grid of warps 0.065 us; the lane launch's last warps add 6-10 ms.  So
+// warps win below about 7,000 bodies, and on short spans as long as the extra
+// throughput of lanes does not pay for those last warps (12,000 bodies over a
+// year: 21 ms against 35; 30,000 over 120 days: 19 against 16.5; 757,000 over
+// 60 days: 260 against 104).  The steps of a body are taken as 3 to start plus
+// one in 14 days.  Mixed precision: lanes are about twice as fast.
+constexpr int64_t kWarpBodies = 8192;
+static bool takes_warps(int64_t n, double span, bool mixed)
+{
+    const double steps = (double)n * (3.0 + std::fabs(span) / 14.0);
+    return n <= (mixed ? kWarpBodies / 2 : kWarpBodies) || steps <= (mixed ? 150e3 : 300e3);
+}
+
+// Bodies that need far more steps than the rest would set the time of a whole
+// launch: past this many attempts they finish with one warp each.  (250,000
+// mixed bodies over a year: 24 + span / 4 days 415 ms, 6 + span / 10 300 ms;
+// the main belt takes 22-26 steps a year.)
+static int attempts_budget(double span) { return 6 + (int)std::min(1e6, std::fabs(span) / 10.0); }
+
+// One propagation launch (and the set-aside bodies' second one) of the chain
+// state along stops (device) with the context's variant for F's precision.
+static int propagate_launch(kete_ctx *ctx, const ForceDev &F, ChainState cs, double t_start,
+                            double t_end, const double *stops_dev, const int32_t *row, int n_stops,
+                            double *out, int64_t stride, bool keep_on_fail, const GridDev *grid,
+                            bool out_aos)
 {
     PropVariant var = ctx->var[F.precision == KETE_MIXED ? 1 : 0];
     unsigned long long *next = nullptr;
     if (var.kind == PROP_WORK_STEALING) GET(S_NEXTBODY, 1, next);
     PropDefer defer{}, *dp = nullptr;
-    if (var.split > 1 && var.budget > 0) {
-        unsigned long long *cnt;
+    // (not on a grid of single-unit legs: a set-aside body would step past them)
+    if (!(grid && grid->n_len == 1 && grid->J > 1) && warp_model(ctx->E, F, defer.model)) {
         GET(S_DEFER_LIST, cs.n, defer.list);
-        GET(S_DEFER_CNT, 2, cnt);
-        defer.count = cnt;
-        defer.next = cnt + 1;
+        GET(S_DEFER_CNT, 1, defer.count);
+        defer.budget0 = var.budget > 0 ? 0 : attempts_budget(t_end - t_start);
         dp = &defer;
     }
     int32_t *order = nullptr;
     unsigned long long *order_n = nullptr;
     if (var.order) {
-        int r = cost_order(ctx, cs.w, cs.n, cs.w + 6 * cs.n, cs.n, stops_dev, n_stops, nullptr,
-                           F.nongrav, &order, &order_n);
+        int r = cost_order(ctx, cs.w, cs.n, cs.w + 6 * cs.n, cs.n, t_end, nullptr, F.nongrav,
+                           &order, &order_n);
         if (r != KETE_OK) return r;
     }
-    ctx->stats.prop_kind = var.kind;
-    ctx->stats.prop_block = var.block;
-    ctx->stats.prop_split = var.split;
-    ctx->stats.prop_budget = var.budget;
-    ctx->stats.prop_order = var.order;
-    CUDA_TRY(launch_propagate(ctx->E, F, cs, stops_dev, n_stops, out, stride, keep_on_fail,
-                              ctx->d_ctr, ctx->stream, nt, leg0, var, next, dp, order, order_n,
+    CUDA_TRY(launch_propagate(ctx->E, F, cs, stops_dev, row, n_stops, out, stride, keep_on_fail,
+                              ctx->d_ctr, ctx->stream, grid, var, next, dp, order, order_n,
                               out_aos));
     if (dp) ctx->extra_launches += 1;   // the second phase
     return KETE_OK;
 }
 
-// Planet states at the Gauss-Radau node epochs of every leg of a chain of stops.
-static int node_table(kete_ctx *ctx, const double *stops_dev, int n_stops, const double *epochs,
-                      NodeTable &nt)
+// Step lengths of a grid, in units of about a day: every whole number up to 16
+// (the main belt's steps are 10-25 days, so rounding a proposal down costs a
+// few per cent of it), then about 10-25 % apart.
+static const int kGridLen[kGridLens] = {1,  2,  3,  4,  5,  6,  7,  8,  9,  10, 11, 12, 13,
+                                        14, 15, 16, 18, 20, 22, 24, 28, 32, 40, 48, 64};
+constexpr int kGridUnits = 512;   // units of one grid: 512 x 25 steps x 9 bodies are 66 MB of rows
+
+// The grid of one launch: points pts[0..J] (host, monotonic).  single: steps
+// of one unit only.
+static int make_grid(kete_ctx *ctx, const std::vector<double> &pts, double unit, bool single,
+                     GridDev &Q)
 {
-    const int nb = ctx->E.n_bodies;
-    double *t0, *h, *r64;
+    const int J = (int)pts.size() - 1;
+    Q = GridDev{};
+    Q.J = J;
+    Q.nb = ctx->E.n_bodies;
+    Q.dir = pts[J] >= pts[0] ? 1 : -1;
+    Q.inv_unit = 1.0 / unit;
+    Q.n_len = 0;
+    for (int q = 0; q < (single ? 1 : kGridLens) && kGridLen[q] <= J; q++)
+        Q.len[Q.n_len++] = kGridLen[q];
+    const size_t steps = (size_t)J * Q.n_len, elems = steps * 8 * Q.nb * 6;
+    double *g, *r64;
     float *r32;
-    GET(S_NT_T0, n_stops, t0);
-    GET(S_NT_H, n_stops, h);
-    GET(S_NT_R64, (size_t)n_stops * 8 * nb * 6, r64);
-    GET(S_NT_R32, (size_t)n_stops * 8 * nb * 6, r32);
-    CUDA_TRY(launch_node_table(ctx->E, stops_dev, n_stops, epochs, t0, h, r64, r32, ctx->stream));
-    nt.t0 = t0;
-    nt.h = h;
-    nt.row64 = r64;
-    nt.row32 = r32;
-    nt.n_legs = n_stops;
-    nt.nb = nb;
+    uint8_t *ok;
+    GET(S_GRID, J + 1, g);
+    GET(S_GRID_R64, elems, r64);
+    GET(S_GRID_R32, elems, r32);
+    GET(S_GRID_OK, steps, ok);
+    CUDA_TRY(cudaMemcpyAsync(g, pts.data(), (J + 1) * sizeof(double), cudaMemcpyHostToDevice,
+                             ctx->stream));
+    Q.g = g;
+    Q.row64 = r64;
+    Q.row32 = r32;
+    Q.ok = ok;
+    CUDA_TRY(launch_grid_rows(ctx->E, Q, r64, r32, ok, ctx->stream));
+    ctx->extra_launches += 1;
+    return KETE_OK;
+}
+
+// Propagate the chain state along the stops (host), stop k to row k of out.
+// t_from: the first body's epoch, or where an earlier call left the chain
+// (NaN: not known).  use_grid: follow a step grid from t_from (from the first
+// stop where t_from is not known or lies past it) in units of about a day;
+// leg_days > 0: the grid's unit, its steps of one unit only.  Marks between
+// stops far apart cut the span into launches of at most kGridUnits units.
+static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const double *stops,
+                     int n_stops, double t_from, double *out, int64_t stride, bool keep_on_fail,
+                     bool use_grid, double leg_days = 0.0, bool out_aos = false)
+{
+    std::vector<double> mark(stops, stops + n_stops);
+    std::vector<int32_t> row((size_t)n_stops);
+    for (int k = 0; k < n_stops; k++) row[k] = k;
+    double *d_stops;
+    int32_t *d_row;
+    const PropVariant &var = ctx->var[F.precision == KETE_MIXED ? 1 : 0];
+    ctx->stats.prop_kind = var.kind;
+    ctx->stats.prop_block = var.block;
+    ctx->stats.prop_split = var.split;
+    ctx->stats.prop_budget = var.budget;
+    ctx->stats.prop_order = var.order;
+    WarpModel model;
+    const bool few = takes_warps(cs.n, stops[n_stops - 1] - t_from, F.precision == KETE_MIXED) &&
+                     var.budget == 0 && leg_days == 0.0 && F.max_iter >= 8 &&
+                     warp_model(ctx->E, F, model);
+    if (few) use_grid = false;
+    const double unit = leg_days > 0.0 ? leg_days : 1.0;
+    double start = t_from;
+    const bool forward = n_stops > 1 ? stops[n_stops - 1] > stops[0] : stops[0] > t_from;
+    if (use_grid && (!std::isfinite(t_from) || (n_stops > 1 && t_from > stops[0]))) start = stops[0];
+    if (use_grid && !(stops[n_stops - 1] != start)) use_grid = false;
+    if (use_grid) {
+        // internal marks where a gap exceeds one launch
+        std::vector<double> m2;
+        std::vector<int32_t> r2;
+        double prev = start;
+        for (int k = 0; k < n_stops; k++) {
+            const double gap = stops[k] - prev, most = unit * kGridUnits;
+            const int64_t parts = (int64_t)std::ceil(std::fabs(gap) / most);
+            for (int64_t p = 1; p < parts; p++) {
+                // on the leg grid, where there is one
+                const double step = leg_days > 0.0 ? (gap > 0 ? most : -most) : gap / (double)parts;
+                m2.push_back(prev + step * (double)p);
+                r2.push_back(-1);
+            }
+            m2.push_back(stops[k]);
+            r2.push_back(k);
+            prev = stops[k];
+        }
+        mark.swap(m2);
+        row.swap(r2);
+    }
+    const int n_marks = (int)mark.size();
+    GET(S_STOPS, n_marks, d_stops);
+    GET(S_STOPROW, n_marks, d_row);
+    CUDA_TRY(cudaMemcpyAsync(d_stops, mark.data(), n_marks * sizeof(double), cudaMemcpyHostToDevice,
+                             ctx->stream));
+    CUDA_TRY(cudaMemcpyAsync(d_row, row.data(), n_marks * sizeof(int32_t), cudaMemcpyHostToDevice,
+                             ctx->stream));
+    if (few) {
+        CUDA_TRY(launch_propagate_warp(ctx->E, F, model, cs, d_stops, d_row, n_marks, out, stride,
+                                       keep_on_fail, ctx->d_ctr, ctx->stream, PropQueue{}, out_aos));
+        return KETE_OK;
+    }
+    if (!use_grid)
+        return propagate_launch(ctx, F, cs, t_from, stops[n_stops - 1], d_stops, d_row, n_marks, out, stride,
+                                keep_on_fail, nullptr, out_aos);
+    for (int k0 = 0; k0 < n_marks;) {
+        int k1 = k0 + 1;   // the marks of this launch
+        while (k1 < n_marks && std::fabs(mark[k1] - start) <= unit * kGridUnits * (1.0 + 1e-12)) k1++;
+        const double end = mark[k1 - 1], span = std::fabs(end - start);
+        GridDev Q;
+        const bool grid = end != start;
+        if (grid) {
+            const int J = (int)std::max(1.0, std::min((double)kGridUnits, std::ceil(span / unit - 1e-9)));
+            const double u = leg_days > 0.0 ? leg_days : span / J;
+            std::vector<double> pts((size_t)J + 1);
+            for (int j = 0; j <= J; j++) pts[j] = start + (forward ? u : -u) * j;
+            pts[J] = end;
+            const int r = make_grid(ctx, pts, u, leg_days > 0.0, Q);
+            if (r != KETE_OK) return r;
+        }
+        const int r = propagate_launch(ctx, F, cs, start, end, d_stops + k0, d_row + k0, k1 - k0, out, stride,
+                                       keep_on_fail, grid ? &Q : nullptr, out_aos);
+        if (r != KETE_OK) return r;
+        if (k1 < n_marks) ctx->extra_launches += 1;
+        start = end;
+        k0 = k1;
+    }
+    return KETE_OK;
+}
+
+// the first body's epoch (device)
+static int first_epoch(kete_ctx *ctx, const double *epochs, double &e0)
+{
+    CUDA_TRY(cudaMemcpyAsync(&e0, epochs, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    CUDA_TRY(cudaStreamSynchronize(ctx->stream));
     return KETE_OK;
 }
 
@@ -556,14 +685,10 @@ extern "C" int kete_propagate(kete_ctx *ctx, double *states, double *epochs, int
         ChainState cs;
         r = run_chain(ctx, F, states, epochs, n, cs);
         if (r != KETE_OK) return r;
-        double *d_stop;
-        GET(S_STOPS, 1, d_stop);
-        CUDA_TRY(cudaMemcpyAsync(d_stop, &t_target, sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
-        NodeTable nt;
-        r = node_table(ctx, d_stop, 1, epochs, nt);
-        if (r != KETE_OK) return r;
         prop_event(ctx, true);
-        r = propagate(ctx, F, cs, d_stop, 1, states, n, true, &nt, 0);
+        double e0;
+        if ((r = first_epoch(ctx, epochs, e0)) != KETE_OK) return r;
+        r = propagate(ctx, F, cs, &t_target, 1, e0, states, n, true, true);
         if (r != KETE_OK) return r;
         prop_event(ctx, false);
         CUDA_TRY(launch_chain_finish(cs, states, epochs, status, ctx->stream));
@@ -598,43 +723,16 @@ extern "C" int kete_propagate_legs(kete_ctx *ctx, double *states, double *epochs
         const double span = t_target - e0;
         const double n_legs = std::ceil(std::fabs(span) / leg_days);
         if (n_legs > 1e7) return fail(ctx, KETE_ERR_BAD_ARG, "more than 10,000,000 legs");
-        const int64_t K = std::max<int64_t>(1, (int64_t)n_legs);
-        std::vector<double> stops((size_t)K);
-        const double sgn = span < 0.0 ? -1.0 : 1.0;
-        for (int64_t k = 0; k + 1 < K; k++) stops[k] = e0 + sgn * leg_days * (double)(k + 1);
-        stops[K - 1] = t_target;
         ChainState cs;
         r = run_chain(ctx, F, states, epochs, n, cs);
         if (r != KETE_OK) return r;
-        double *d_stops;
-        GET(S_STOPS, K, d_stops);
-        CUDA_TRY(cudaMemcpyAsync(d_stops, stops.data(), K * sizeof(double), cudaMemcpyHostToDevice,
-                                 ctx->stream));
-        // internal stops in chunks whose states go to scratch (at most 2 GiB),
-        // then the target alone, whose states go to the caller's array: a body
-        // that failed is not written there and keeps its input state
-        const int64_t M = K - 1;
-        const int64_t cap = std::max<int64_t>(1, ((int64_t)1 << 31) / (48 * n));
-        const int64_t C = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(M, 512), cap));
-        double *scratch = nullptr;
-        if (M > 0) GET(S_LEG_OUT, (size_t)C * 6 * (size_t)n, scratch);
-        int launches = 2;
         prop_event(ctx, true);
-        for (int64_t j0 = 0; j0 < K;) {
-            const bool last = (j0 == M);
-            const int64_t cnt = last ? 1 : std::min(C, M - j0);
-            NodeTable nt;
-            r = node_table(ctx, d_stops + j0, (int)cnt, j0 == 0 ? epochs : d_stops + j0 - 1, nt);
-            if (r != KETE_OK) return r;
-            r = propagate(ctx, F, cs, d_stops + j0, (int)cnt, last ? states : scratch, n, true, &nt,
-                          0);
-            if (r != KETE_OK) return r;
-            launches += 2;
-            j0 += cnt;
-        }
+        r = propagate(ctx, F, cs, &t_target, 1, e0, states, n, true, true,
+                      n_legs > 1.0 ? leg_days : 0.0);   // one leg: as kete_propagate
+        if (r != KETE_OK) return r;
         prop_event(ctx, false);
         CUDA_TRY(launch_chain_finish(cs, states, epochs, status, ctx->stream));
-        ctx->stats.launches = launches;
+        ctx->stats.launches = 3;
     }
     r = stats_end(ctx);
     if (r != KETE_OK) return r;
@@ -663,14 +761,10 @@ extern "C" int kete_propagate_stops(kete_ctx *ctx, const double *states, const d
         ChainState cs;
         r = run_chain(ctx, F, states, epochs, n, cs);
         if (r != KETE_OK) return r;
-        double *d_stops;
-        GET(S_STOPS, n_stops, d_stops);
-        CUDA_TRY(cudaMemcpyAsync(d_stops, stops, n_stops * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
-        NodeTable nt;
-        r = node_table(ctx, d_stops, (int)n_stops, epochs, nt);
-        if (r != KETE_OK) return r;
         prop_event(ctx, true);
-        r = propagate(ctx, F, cs, d_stops, (int)n_stops, out, n, false, &nt, 0);
+        double e0;
+        if ((r = first_epoch(ctx, epochs, e0)) != KETE_OK) return r;
+        r = propagate(ctx, F, cs, stops, (int)n_stops, e0, out, n, false, true);
         if (r != KETE_OK) return r;
         prop_event(ctx, false);
         CUDA_TRY(launch_chain_finish(cs, nullptr, nullptr, status, ctx->stream));
@@ -875,7 +969,11 @@ static int fov_check_impl(kete_ctx *ctx, const double *states, const double *epo
     CUDA_TRY(cudaStreamSynchronize(st));
     const int32_t nb = h_nb;
     std::vector<int32_t> h_first(nb + 1);
+    std::vector<double> h_tref(nb);
+    double chain_at = 0.0;   // where the chain of midpoints stands
     CUDA_TRY(cudaMemcpyAsync(h_first.data(), B.first, (nb + 1) * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaMemcpyAsync(h_tref.data(), B.t_ref, nb * sizeof(double), cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaMemcpyAsync(&chain_at, epochs, sizeof(double), cudaMemcpyDeviceToHost, st));
     GET(S_BO, 3 * nb, B.O);
     GET(S_BROBS, nb, B.robs);
     GET(S_BTSPAN, nb, B.tspan);
@@ -920,10 +1018,7 @@ static int fov_check_impl(kete_ctx *ctx, const double *states, const double *epo
     kete_hit *hit_tmp;
     GET(S_HITTMP, hit_cap, hit_tmp);
     hit_cap = ctx->slot[S_HITTMP].bytes / sizeof(kete_hit);
-    NodeTable nt;
-    r = node_table(ctx, B.t_ref, nb, epochs, nt);
-    if (r != KETE_OK) return r;
-    launches++;
+    CUDA_TRY(cudaStreamSynchronize(st));
     unsigned long long hits_total = 0, cands_total = 0, exact_total = 0;
     for (int32_t k0 = 0; k0 < nb; k0 += C) {
         const int32_t k1 = std::min(nb, k0 + C), nk = k1 - k0;
@@ -931,8 +1026,10 @@ static int fov_check_impl(kete_ctx *ctx, const double *states, const double *epo
         const int32_t nek = e1 - e0;
         // propagation to the batch midpoints of this chunk
         prop_event(ctx, true);
-        r = propagate(ctx, F, cs, B.t_ref + k0, nk, stop_states, n, false, &nt, k0, true);
+        r = propagate(ctx, F, cs, h_tref.data() + k0, nk, chain_at, stop_states, n, false, true, 0.0,
+                      true);
         if (r != KETE_OK) return r;
+        chain_at = h_tref[k1 - 1];
         prop_event(ctx, false);
         launches++;
         // exposures of the chunk into sky cells
@@ -1199,12 +1296,11 @@ extern "C" int kete_autotune(kete_ctx *ctx, const double *states, const double *
     // be dominated by its longest-lived ones, which favours the split variants.
     const int64_t m = std::min(n, max_sample);
     const double scale = (double)m / (double)n;
-    double *sst, *sep, *out, *d_stops;
+    double *sst, *sep, *out, e_first;
     GET(S_TUNE_ST, 6 * m, sst);
     GET(S_TUNE_EP, m, sep);
     GET(S_TUNE_OUT, (size_t)n_stops * 6 * m, out);
-    GET(S_STOPS, n_stops, d_stops);
-    CUDA_TRY(cudaMemcpyAsync(d_stops, stops, n_stops * sizeof(double), cudaMemcpyHostToDevice, st));
+    if ((r = first_epoch(ctx, epochs, e_first)) != KETE_OK) return r;
     CUDA_TRY(launch_gather_bodies(states, epochs, n, m, sst, sep, st));
     // schedules x cost order, then the split variants (with cost order)
     PropVariant cands[9];
@@ -1237,12 +1333,9 @@ extern "C" int kete_autotune(kete_ctx *ctx, const double *states, const double *
             ChainState cs;
             int r2 = run_chain(ctx, F, st_, ep_, cnt, cs);
             if (r2 != KETE_OK) return r2;
-            NodeTable nt;
-            r2 = node_table(ctx, d_stops, (int)n_stops, ep_, nt);
-            if (r2 != KETE_OK) return r2;
             CUDA_TRY(cudaMemsetAsync(ctx->d_ctr, 0, sizeof(DevCounters), st));
             CUDA_TRY(cudaEventRecord(e0, st));
-            r2 = propagate(ctx, F, cs, d_stops, (int)n_stops, out_, cnt, false, &nt, 0);
+            r2 = propagate(ctx, F, cs, stops, (int)n_stops, e_first, out_, cnt, false, true);
             if (r2 != KETE_OK) return r2;
             CUDA_TRY(cudaEventRecord(e1, st));
             CUDA_TRY(cudaEventSynchronize(e1));
@@ -1392,7 +1485,7 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
                 CUDA_TRY(launch_adjoint_last_epoch(P, i0, nc, t_end, ctx->stream));
                 // bodies with and without non-gravitational terms in separate
                 // ranges, so that the full-model records rarely share a warp
-                int r2 = cost_order(ctx, states + i0, n, epochs + i0, nc, nullptr, 0, t_end,
+                int r2 = cost_order(ctx, states + i0, n, epochs + i0, nc, 0.0, t_end,
                                     F.nongrav ? F.nongrav + i0 : nullptr, &order, &order_n);
                 if (r2 != KETE_OK) return r2;
                 launches += 1;

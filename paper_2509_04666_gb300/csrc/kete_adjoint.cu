@@ -557,7 +557,6 @@ k_adj_forward(EphemDev E, ForceDev F, AdjBuffers B, AdjProblem P, int64_t i0, in
     S.have_a0 = false;
     S.ng = nullptr;   // set per body on the full-model path
     S.ng_chi = 0.0;
-    const LegView L = leg_view(nullptr, 0);
     double *rec = nullptr, *recx = nullptr;   // recx: null for a body without terms
     bool first = true;
     for (;;) {
@@ -641,7 +640,7 @@ k_adj_forward(EphemDev E, ForceDev F, AdjBuffers B, AdjProblem P, int64_t i0, in
                 if (RICH && recx) {   // the accepted attempt's coefficients give the node states
                     const double x0[3] = {x[0], x[1], x[2]}, v0[3] = {v[0], v[1], v[2]};
                     Attempt A;
-                    status = step_begin<KETE_FP64, true>(E, F, L, x, v, t, dt, ts, S, A, cnt, r + 2);
+                    status = step_begin<KETE_FP64, true>(E, F, x, v, t, dt, ts, S, A, cnt, r + 2);
                     while (status == KETE_BODY_OK) {
                         bool done = false;
                         status = attempt_sweep<KETE_FP64, true>(E, F, t, x, v, S.a0, S.as0,
@@ -655,7 +654,7 @@ k_adj_forward(EphemDev E, ForceDev F, AdjBuffers B, AdjProblem P, int64_t i0, in
                         status = record_extra(E, F, t_prev, x0, v0, S.a0, A, S.ng,
                                               recx + (size_t)slot * kAdjRecX);
                 } else {
-                    status = step_once<KETE_FP64, true>(E, F, L, x, v, t, dt, ts, S, cnt, r + 2);
+                    status = step_once<KETE_FP64, true>(E, F, x, v, t, dt, ts, S, cnt, r + 2);
                 }
                 if (status == KETE_BODY_OK && t != t_prev) {
                     r[0] = t_prev;

@@ -117,38 +117,6 @@ __device__ __forceinline__ const double *ephem_coef(const EphemDev &E, int body,
 }
 
 // ---------------------------------------------------------------------------
-// Lane groups: G consecutive lanes (G a power of two, <= 32) integrating one
-// body together.  Every lane of a group holds the same integrator state and
-// runs the same control flow; in a force evaluation lane `rank` takes the
-// masses m = rank, rank + G, ... and the partial sums are combined by a
-// butterfly of shuffles, which leaves the same bits in every lane (each pair
-// adds the same two values).  G = 1 is the plain one-lane-per-body form.
-// ---------------------------------------------------------------------------
-template <int G>
-struct LaneGroup {
-    static_assert(G == 1 || G == 2 || G == 4 || G == 8 || G == 16 || G == 32, "G");
-    __device__ __forceinline__ static int rank() { return G == 1 ? 0 : (int)(threadIdx.x & (G - 1)); }
-    __device__ __forceinline__ static unsigned mask()
-    {
-        if (G == 32) return 0xffffffffu;
-        return ((1u << G) - 1u) << ((threadIdx.x & 31) & ~(unsigned)(G - 1));
-    }
-    template <typename T>
-    __device__ __forceinline__ static T sum(T v)
-    {
-#pragma unroll
-        for (int o = G / 2; o >= 1; o /= 2) v += __shfl_xor_sync(mask(), v, o);
-        return v;
-    }
-    __device__ __forceinline__ static uint32_t bit_or(uint32_t v)
-    {
-#pragma unroll
-        for (int o = G / 2; o >= 1; o /= 2) v |= __shfl_xor_sync(mask(), v, o);
-        return v;
-    }
-};
-
-// ---------------------------------------------------------------------------
 // Force model (Eq. A.1): for each active mass m with r = x - x_m, v = v - v_m:
 //   Newton  -mu r / |r|^3
 //   GR      mu / (c^2 |r|^3) [ (4 mu/|r| - |v|^2) r + 4 (r.v) v ]       (Eq. A.3)
@@ -396,28 +364,6 @@ struct Encounter {
     double d0[3];     // x0 - p_m(t0)
 };
 
-// the group's nearest candidate (ties to the lower table index, as the
-// one-lane loop over m in order)
-template <int G>
-__device__ __forceinline__ void encounter_reduce(double &best, Encounter &enc)
-{
-#pragma unroll
-    for (int o = G / 2; o >= 1; o /= 2) {
-        const unsigned gm = LaneGroup<G>::mask();
-        const double ob = __shfl_xor_sync(gm, best, o);
-        const int om = __shfl_xor_sync(gm, enc.m, o);
-        double od[3];
-#pragma unroll
-        for (int c = 0; c < 3; c++) od[c] = __shfl_xor_sync(gm, enc.d0[c], o);
-        if (ob < best || (ob == best && om < enc.m)) {
-            best = ob;
-            enc.m = om;
-#pragma unroll
-            for (int c = 0; c < 3; c++) enc.d0[c] = od[c];
-        }
-    }
-}
-
 // Node rows: planet states at one Gauss-Radau node epoch of a batch leg,
 // shared by every body whose step spans that whole leg.
 //   row64[m*6 + 0..5]  barycentric position, velocity (FP64)
@@ -449,41 +395,18 @@ struct NgOut {
     int status;
     double chi;   // the thermal lag's two-body solution (universal anomaly), for the next call
 };
-static __device__ __noinline__ NgOut nongrav_terms(const EphemDev &E, const double *row64, Seg g,
-                                                   const kete_nongrav *P, double x0, double x1,
-                                                   double x2, double v0, double v1, double v2,
-                                                   double chi0);
-
-// Lane groups (G > 1): the body's non-gravitational terms (ng may be null)
-// computed by the group's last lane -- the one that holds the fewest masses
-// -- and added to its partial sum acc before the group sum; every lane of
-// the group returns the same status.
-template <int G>
-__device__ __forceinline__ int group_nongrav(const EphemDev &E, const double *row64, Seg g,
-                                             const kete_nongrav *ng, const double x[3],
-                                             const double v[3], double acc[3], double *ng_chi)
-{
-    if (!ng) return KETE_BODY_OK;
-    int st = KETE_BODY_OK;
-    if (LaneGroup<G>::rank() == G - 1) {
-        const NgOut o = nongrav_terms(E, row64, g, ng, x[0], x[1], x[2], v[0], v[1], v[2],
-                                      ng_chi ? *ng_chi : 0.0);
-        if (ng_chi) *ng_chi = o.chi;
-        st = o.status;
-        acc[0] += o.a[0];
-        acc[1] += o.a[1];
-        acc[2] += o.a[2];
-    }
-    return __shfl_sync(LaneGroup<G>::mask(), st, G - 1, G);
-}
+static __device__ __forceinline__ NgOut nongrav_terms(const EphemDev &E, const double *row64, Seg g,
+                                                      const kete_nongrav *P, double x0, double x1,
+                                                      double x2, double v0, double v1, double v2,
+                                                      double chi0);
 
 // Full-FP64 acceleration.
 // detect (step start, off = 0): also record in enc the nearest planet within
 // kEncounterAu and its relative position; otherwise enc is read.
 // JAC: also return in J the Newtonian da/dx (see newton_jacobian), from the
-// same relative vectors as the force.  G: lanes per body (see LaneGroup).
+// same relative vectors as the force.
 // ng: the body's non-gravitational terms (null: none), added after the sum.
-template <bool JAC = false, int G = 1>
+template <bool JAC = false>
 __device__ __forceinline__ int accel_fp64(const EphemDev &E, const ForceDev &F, double t0,
                                           double off, const double *__restrict__ row64,
                                           const double x[3], const double v[3], double a[3],
@@ -512,7 +435,7 @@ __device__ __forceinline__ int accel_fp64(const EphemDev &E, const ForceDev &F, 
     const bool use_basis = !row64 && E.n_coef <= kBasisMax && threadIdx.x < kBasisLanes &&
                            blockDim.x <= kBasisLanes;
     if (use_basis) cheb_basis(E.n_coef, g.tau, (F.gr_mask & F.active_mask) != 0u, basis);
-    for (int m = LaneGroup<G>::rank(); m < E.n_bodies; m += G) {
+    for (int m = 0; m < E.n_bodies; m++) {
         if (!((F.active_mask >> m) & 1u)) continue;
         const bool gr = (F.gr_mask >> m) & 1u, j2 = (F.j2_mask >> m) & 1u;
         double st[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
@@ -555,20 +478,6 @@ __device__ __forceinline__ int accel_fp64(const EphemDev &E, const ForceDev &F, 
         mass_terms<double>(mass_k64(E, F, m), true, gr, j2, r, w, a);
         if (JAC) newton_jacobian(E.gm[m], r, J);
     }
-    if (G > 1) {
-        // the body's own terms go to the group's last lane, which holds the
-        // fewest masses, and join the group sum (a lagged comet term costs a
-        // two-body solve: done once per group, beside the others' masses)
-        const int ng_status = group_nongrav<G>(E, row64, g, ng, x, v, a, ng_chi);
-#pragma unroll
-        for (int c = 0; c < 3; c++) a[c] = LaneGroup<G>::sum(a[c]);
-        if (JAC) {
-#pragma unroll
-            for (int q = 0; q < 6; q++) J[q] = LaneGroup<G>::sum(J[q]);
-        }
-        if (detect) encounter_reduce<G>(best, enc);
-        return ng_status;
-    }
     if (ng) {
         const NgOut o = nongrav_terms(E, row64, g, ng, x[0], x[1], x[2], v[0], v[1], v[2],
                                       ng_chi ? *ng_chi : 0.0);
@@ -594,9 +503,7 @@ constexpr double kCloseAu = 0.1;
 
 // detect (step start, off = 0): planets within 2 kCloseAu go to FP64 and are
 // recorded in `close` (held for the step), and the nearest within kEncounterAu
-// in enc; otherwise close and enc are read.  G: lanes per body (LaneGroup);
-// the Sun's terms belong to rank 0, every lane forms the Sun-relative position.
-template <int G = 1>
+// in enc; otherwise close and enc are read.
 __device__ __forceinline__ int accel_mixed(const EphemDev &E, const ForceDev &F, double t0,
                                            double off, const double *__restrict__ row64,
                                            const float *__restrict__ row32, uint32_t &close,
@@ -642,8 +549,7 @@ __device__ __forceinline__ int accel_mixed(const EphemDev &E, const ForceDev &F,
 #pragma unroll
     for (int c = 0; c < 3; c++) vf[c] = vf_in ? vf_in[c] : (float)v[c];
     float af[3] = {0.f, 0.f, 0.f};
-    const int rk = LaneGroup<G>::rank();
-    if (rk == 0 && (F.active_mask & 1u)) {
+    if (F.active_mask & 1u) {
         // Sun monopole, FP64
         double rr = fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2]));
         double ri = rsqrt(rr);
@@ -666,7 +572,7 @@ __device__ __forceinline__ int accel_mixed(const EphemDev &E, const ForceDev &F,
         for (int q = 0; q < 3; q++) sunf[q] = (float)sun[q];
     }
     const float tau32 = row64 ? 0.f : (float)g.tau;
-    for (int m = (rk == 0 ? G : rk); m < E.n_bodies; m += G) {
+    for (int m = 1; m < E.n_bodies; m++) {
         if (!((F.active_mask >> m) & 1u)) continue;
         const bool gr = (F.gr_mask >> m) & 1u, j2 = (F.j2_mask >> m) & 1u;
         float st[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -718,20 +624,7 @@ __device__ __forceinline__ int accel_mixed(const EphemDev &E, const ForceDev &F,
         float w[3] = {vf[0] - st[3], vf[1] - st[4], vf[2] - st[5]};
         mass_terms<float>(mass_k32(F, m), true, gr, j2, r, w, af);
     }
-    int ng_status = KETE_BODY_OK;
-    if (G > 1) {
-        ng_status = group_nongrav<G>(E, row64, g, ng, x, v, as, ng_chi);   // FP64, smooth part
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            as[c] = LaneGroup<G>::sum(as[c]);
-            af[c] = LaneGroup<G>::sum(af[c]);
-        }
-        if (detect) {
-            close = LaneGroup<G>::bit_or(close);
-            encounter_reduce<G>(best, enc);
-        }
-        if (ng_status != KETE_BODY_OK) return ng_status;
-    } else if (ng) {   // FP64, part of the smooth FP64 sum that controls the step
+    if (ng) {   // FP64, part of the smooth FP64 sum that controls the step
         const NgOut o = nongrav_terms(E, row64, g, ng, x[0], x[1], x[2], v[0], v[1], v[2],
                                       ng_chi ? *ng_chi : 0.0);
         if (ng_chi) *ng_chi = o.chi;
@@ -884,27 +777,17 @@ __device__ __forceinline__ bool kepler_uv(double mu, double sqmu, const double r
     return ok;
 }
 
-// Non-gravitational terms (App. A.4-A.5) of a body at barycentric (x, v):
-// heliocentric r, w from the Sun's state at the same epoch (node row or
-// table), then radiation pressure with drag (Eq. A.6, radial-speed reading)
-// and the JPL comet model (Eq. A.7) from the two-body state dt days earlier.
-static __device__ __noinline__ NgOut nongrav_terms(const EphemDev &E, const double *row64, Seg g,
-                                                   const kete_nongrav *P, double x0, double x1,
-                                                   double x2, double v0, double v1, double v2,
-                                                   double chi0)
+// Non-gravitational terms (App. A.4-A.5) of a body at heliocentric (r, w):
+// radiation pressure with drag (Eq. A.6, radial-speed reading) and the JPL
+// comet model (Eq. A.7) from the two-body state dt days earlier.
+static __device__ __noinline__ NgOut nongrav_helio(double mu, const kete_nongrav *P, double r0,
+                                                   double r1, double r2, double w0, double w1,
+                                                   double w2, double chi0)
 {
     NgOut o = {{0.0, 0.0, 0.0}, KETE_BODY_OK, chi0};
-    double sun[6];
-    if (row64) {
-#pragma unroll
-        for (int q = 0; q < 6; q++) sun[q] = __ldg(row64 + q);
-    } else {
-        cheb_state64(E, 0, g.s, g.tau, sun, true);
-    }
     const kete_nongrav p = *P;
-    const double mu = E.gm[0];
-    const double r[3] = {x0 - sun[0], x1 - sun[1], x2 - sun[2]};
-    const double w[3] = {v0 - sun[3], v1 - sun[4], v2 - sun[5]};
+    const double r[3] = {r0, r1, r2};
+    const double w[3] = {w0, w1, w2};
     if (p.beta != 0.0) {
         const double rr = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
         const double rn = sqrt(rr);
@@ -951,6 +834,24 @@ static __device__ __noinline__ NgOut nongrav_terms(const EphemDev &E, const doub
             o.a[c] += gq * (p.a1 * rh[c] + p.a2 * th[c] + p.a3 * nh[c]);
     }
     return o;
+}
+
+// nongrav_helio of a body at barycentric (x, v), the Sun's state from the
+// node row or the table.
+static __device__ __forceinline__ NgOut nongrav_terms(const EphemDev &E, const double *row64, Seg g,
+                                                      const kete_nongrav *P, double x0, double x1,
+                                                      double x2, double v0, double v1, double v2,
+                                                      double chi0)
+{
+    double sun[6];
+    if (row64) {
+#pragma unroll
+        for (int q = 0; q < 6; q++) sun[q] = __ldg(row64 + q);
+    } else {
+        cheb_state64(E, 0, g.s, g.tau, sun, true);
+    }
+    return nongrav_helio(E.gm[0], P, x0 - sun[0], x1 - sun[1], x2 - sun[2], v0 - sun[3],
+                         v1 - sun[4], v2 - sun[5], chi0);
 }
 
 // RA/Dec (equatorial J2000) of an ecliptic vector

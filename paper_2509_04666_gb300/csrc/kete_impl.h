@@ -38,7 +38,8 @@ struct ForceDev {
     double gm4[KETE_MAX_BODIES], grk[KETE_MAX_BODIES], gr4k[KETE_MAX_BODIES];
     double pole_m2[KETE_MAX_BODIES][3];
     double eps, eps_pc, safety, dt_init;
-    int32_t max_iter, pad;
+    int32_t max_iter;
+    float log2_eps;
     int64_t max_steps;
     // FP32 copies for the mixed-precision planetary terms (rounded once here)
     float gm32[KETE_MAX_BODIES];
@@ -60,14 +61,20 @@ struct DevCounters {
     int pad;
 };
 
-// planet states at the 8 Gauss-Radau node epochs of each leg of a chain of
-// stops (leg k runs from t0[k] to t0[k] + h[k]); h[k] is NaN when the leg
-// cannot use the rows (a node outside the table)
-struct NodeTable {
-    const double *t0, *h;
-    const double *row64;   // [leg][8][n_bodies][6] FP64 barycentric pos, vel
-    const float *row32;    // [leg][8][n_bodies][6] FP32 heliocentric pos, vel
-    int n_legs, nb;
+// Step grid of a propagation: epochs g[0..J] that every body's steps meet, and
+// the planet states at the 8 Gauss-Radau node epochs of the steps g[j] ->
+// g[j + len[q]] (rows of step (j, q) at (j n_len + q) 8 nb 6), shared by every
+// body that takes that step.  ok[j n_len + q] is 0 where a node lies outside
+// the table or the grid.
+constexpr int kGridLens = 25;
+struct GridDev {
+    const double *g;
+    const double *row64;   // [step][8][nb][6] FP64 barycentric pos, vel
+    const float *row32;    // [step][8][nb][6] FP32 heliocentric pos, vel
+    const uint8_t *ok;     // [step]
+    double inv_unit;       // 1 / days per grid unit
+    int J, n_len, nb, dir; // dir: +1 forward in time, -1 backward
+    int len[kGridLens];    // step lengths in grid units, ascending from 1
 };
 
 // per-body working state of a propagation chain: [8][n] = x,y,z,vx,vy,vz,t,dt;
@@ -86,14 +93,25 @@ struct PropQueue {
     int resume = 0;                              // bodies resume at cs.kstop (else stop 0)
     int32_t *defer = nullptr;                    // set-aside bodies are appended here
     unsigned long long *defer_n = nullptr;
-    int budget = 0;                              // step attempts per stop reached
+    int budget = 0;                              // step attempts per stop reached ...
+    int budget0 = 0;                             // ... and besides
 };
 
-// scratch of the two-phase (split) launch
+// Masses by lane of the one-warp-per-body kernel (kete_warp.cu): slot s of lane r (of four)
+// holds body list[4 s + r]; the masses with GR or J2 terms fill slot 0, whose
+// code evaluates both without branches.
+constexpr int kWarpSlots = 3;
+struct WarpModel {
+    int list[4 * kWarpSlots];   // -1: none
+    int gr, j2;                 // any GR / J2 mass
+};
+
+// scratch of the two-phase launch (long bodies set aside)
 struct PropDefer {
     int32_t *list;                 // [n]
     unsigned long long *count;     // set-aside bodies
-    unsigned long long *next;      // work-stealing counter of the second phase
+    int budget0;                   // PropQueue::budget0
+    WarpModel model;               // masses of the second phase
 };
 
 // launch helpers implemented in the .cu files ---------------------------------
@@ -102,9 +120,9 @@ cudaError_t launch_ephem_eval(const EphemDev &E, const double *t, int64_t n, int
                               double *pos, double *vel, cudaStream_t st);
 cudaError_t launch_chain_init(ChainState cs, const double *states, const double *epochs,
                               const ForceDev &F, cudaStream_t st);
-cudaError_t launch_node_table(const EphemDev &E, const double *stops_dev, int n_stops,
-                              const double *epoch0, double *t0, double *h, double *row64,
-                              float *row32, cudaStream_t st);
+// fill the rows and flags of a grid whose points are at grid.g
+cudaError_t launch_grid_rows(const EphemDev &E, const GridDev &grid, double *row64, float *row32,
+                             uint8_t *ok, cudaStream_t st);
 // how the propagation kernel is launched (chosen by the autotuner)
 enum PropKind { PROP_STATIC = 0, PROP_WORK_STEALING = 1 };
 struct PropVariant {
@@ -116,15 +134,27 @@ struct PropVariant {
     double grid_scale = 1.0;   // persistent grids scaled by this (<= 1: a sample of the
                                // bodies run with as many bodies per lane as the whole)
 };
+// stop_row (device, may be null): output row of each stop, -1: not written
+// (null: stop k is row k).  grid (may be null): the step grid to follow.
 cudaError_t launch_propagate(const EphemDev &E, const ForceDev &F, ChainState cs,
-                             const double *stops_dev, int n_stops, double *out,
-                             int64_t out_stride, bool keep_on_fail, DevCounters *ctr,
-                             cudaStream_t st, const NodeTable *nt = nullptr, int leg0 = 0,
+                             const double *stops_dev, const int32_t *stop_row, int n_stops,
+                             double *out, int64_t out_stride, bool keep_on_fail, DevCounters *ctr,
+                             cudaStream_t st, const GridDev *grid = nullptr,
                              PropVariant var = PropVariant{PROP_STATIC, 128},
                              unsigned long long *next_body = nullptr,
                              PropDefer *defer = nullptr, const int32_t *order = nullptr,
                              const unsigned long long *order_n = nullptr, bool out_aos = false);
 int propagate_ws_blocks(int block, int mode);
+// kete_warp.cu: one warp per body.
+// false: the model does not fit (the Sun inactive, more than 12 masses, more
+// than 4 with GR or J2 terms)
+bool warp_model(const EphemDev &E, const ForceDev &F, WarpModel &W);
+cudaError_t upload_warp_tables(cudaStream_t st);
+// q: bodies 0..n-1, or q.list (resuming at their saved stops if q.resume)
+cudaError_t launch_propagate_warp(const EphemDev &E, const ForceDev &F, const WarpModel &W,
+                                  ChainState cs, const double *stops, const int32_t *row,
+                                  int n_stops, double *out, int64_t stride, bool keep_on_fail,
+                                  DevCounters *ctr, cudaStream_t st, PropQueue q, bool out_aos);
 cudaError_t launch_gather_bodies(const double *st, const double *ep, int64_t n, int64_t m,
                                  double *dst, double *dep, cudaStream_t s);
 cudaError_t launch_chain_finish(ChainState cs, double *states, double *epochs,

@@ -95,7 +95,7 @@ int noalloc_propagate(int device, cudaStream_t st, const EphemDev &E, const Forc
         return KETE_ERR_CUDA;
     }
     if ((e = launch_chain_init(cs, states, epochs, F, st)) == cudaSuccess &&
-        (e = launch_propagate(E, F, cs, &s->stop, 1, states, n, true, &s->ctr, st)) == cudaSuccess)
+        (e = launch_propagate(E, F, cs, &s->stop, nullptr, 1, states, n, true, &s->ctr, st)) == cudaSuccess)
         e = launch_chain_finish(cs, states, epochs, status, st);
     if (e != cudaSuccess) {
         *why = cudaGetErrorString(e);

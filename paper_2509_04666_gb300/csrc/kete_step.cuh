@@ -82,20 +82,19 @@ struct Cnt {
     unsigned long long steps, rejected, evals, iters, node_evals;
 };
 
-// Rows of the node table for leg kg, or null when the step (t, h) does not span
-// that whole leg.
-struct LegRows {
+// Planet rows of the 8 nodes of one step (null: the planets are summed per
+// thread).
+struct StepRows {
     const double *r64;
     const float *r32;
-    int stride64;   // doubles per node
+    int stride;   // elements per node
 };
 
 // Force evaluation dispatch by precision mode.
 // detect: the evaluation at a step start, which also finds the planets near
 // the body (see accel_fp64 / accel_mixed).
 // JAC (FP64 only): also store the Newtonian da/dx at this point to jout[0..5].
-// G: lanes per body (LaneGroup).
-template <int MODE, bool JAC = false, int G = 1>
+template <int MODE, bool JAC = false>
 __device__ __forceinline__ int accel(const EphemDev &E, const ForceDev &F, double t0, double off,
                                      const double *row64, const float *row32, uint32_t &close,
                                      const double x[3], const double v[3], double a[3],
@@ -105,10 +104,10 @@ __device__ __forceinline__ int accel(const EphemDev &E, const ForceDev &F, doubl
 {
     static_assert(!(JAC && MODE == KETE_MIXED), "Jacobian capture is FP64 only");
     if (MODE == KETE_MIXED)
-        return accel_mixed<G>(E, F, t0, off, row64, row32, close, x, v, a, as, enc, dx, detect, ng,
+        return accel_mixed(E, F, t0, off, row64, row32, close, x, v, a, as, enc, dx, detect, ng,
                               vf, ng_chi);
     double J[6];
-    int st = accel_fp64<JAC, G>(E, F, t0, off, row64, x, v, a, enc, dx, detect, J, ng, ng_chi);
+    int st = accel_fp64<JAC>(E, F, t0, off, row64, x, v, a, enc, dx, detect, J, ng, ng_chi);
     as[0] = a[0]; as[1] = a[1]; as[2] = a[2];
     if (JAC) {
 #pragma unroll
@@ -119,19 +118,19 @@ __device__ __forceinline__ int accel(const EphemDev &E, const ForceDev &F, doubl
 
 // Corrector state of one Gauss-Radau step attempt of size h (from t to
 // t_new) between corrector sweeps; one sweep is one corrector iteration over
-// the 7 substep nodes.  rows.r64 != null: the step spans the whole leg and
-// the planets come from the node rows (node n at rows.r64 + n * stride).
+// the 7 substep nodes.  rows.r64 != null: a grid step, the planets come from
+// its rows (node n at rows.r64 + n * stride).
 struct Attempt {
     double b[7][3], g[7][3];
     float bf[7][3];         // mixed precision: b in FP32, for the node velocity
     double gs7[3];          // mixed precision: b6 of the FP64 part, last sweep
     double amax, pc_prev;   // max|a| at the last node and the last convergence measure
     double h, t_new;
-    LegRows rows;
+    StepRows rows;
     int it;                 // sweeps done
 };
 
-__device__ __forceinline__ void attempt_begin(Attempt &A, double h, double t_new, LegRows rows)
+__device__ __forceinline__ void attempt_begin(Attempt &A, double h, double t_new, StepRows rows)
 {
 #pragma unroll
     for (int m = 0; m < 7; m++)
@@ -180,7 +179,7 @@ __device__ __forceinline__ void node_update(Attempt &A, const double Fn[3], cons
 // (max|db6|/max|a| < eps_pc), stopped improving (from the third sweep) or
 // reached max_iter sweeps.  JAC: every node evaluation also stores da/dx at
 // node n to jrec[6n..6n+5]; the last sweep's values remain.
-template <int MODE, bool JAC = false, int G = 1, bool V32 = false>
+template <int MODE, bool JAC = false, bool V32 = false>
 __device__ __forceinline__ int attempt_sweep(const EphemDev &E, const ForceDev &F, double t,
                                              const double x0[3], const double v0[3],
                                              const double a0[3], const double as0[3],
@@ -243,9 +242,9 @@ __device__ __forceinline__ int attempt_sweep(const EphemDev &E, const ForceDev &
             }
         }
         double Fn[3], Fs[3];
-        const double *r64 = A.rows.r64 ? A.rows.r64 + n * A.rows.stride64 : nullptr;
-        const float *r32 = A.rows.r32 ? A.rows.r32 + n * A.rows.stride64 : nullptr;
-        int st = accel<MODE, JAC, G>(E, F, t, sh, r64, r32, close, xn, vn, Fn, Fs, enc, dxn,
+        const double *r64 = A.rows.r64 ? A.rows.r64 + n * A.rows.stride : nullptr;
+        const float *r32 = A.rows.r32 ? A.rows.r32 + n * A.rows.stride : nullptr;
+        int st = accel<MODE, JAC>(E, F, t, sh, r64, r32, close, xn, vn, Fn, Fs, enc, dxn,
                                      false, JAC ? jrec + 6 * n : nullptr, ng,
                                      vel32 ? vnf : nullptr, ng_chi);
         cnt.evals++;
@@ -320,107 +319,208 @@ struct StepState {
     double a0[3], as0[3];   // acceleration at the step start (and its FP64 part)
     uint32_t close;         // planets near the body at the step start (mixed precision)
     Encounter enc;          // nearest planet within kEncounterAu (close-encounter path)
-    double t_stop;          // end of the step's range: the target, or the next table
-                            // segment boundary during an encounter
+    double bound;           // epoch no step may pass: the next table segment boundary
+                            // during an encounter, else infinite
     bool have_a0;           // a0 valid for (x, v, t): kept across a rejection
     const kete_nongrav *ng; // the body's non-gravitational terms (null: none)
     double ng_chi;          // the thermal lag's last two-body solution (0: none yet)
 };
 
-// Node-table view of leg kg (null pointers: no rows).
-struct LegView {
-    double t0, h;
-    const double *r64;
-    const float *r32;
-    int stride;
-};
-
-__device__ __forceinline__ LegView leg_view(const NodeTable *nt, int kg)
+// The acceleration at the start of a step attempt of (x, v, t) if it is not
+// known yet (kept across a rejection), from node-0 rows when given, and the
+// epoch no step toward `dir` may pass: during an encounter no step straddles
+// a boundary of the planet polynomials (S.bound; infinite otherwise).
+template <int MODE, bool JAC>
+__device__ __forceinline__ int step_start(const EphemDev &E, const ForceDev &F, const double *r64,
+                                          const float *r32, const double x[3], const double v[3],
+                                          double t, bool forward, StepState &S, Cnt &cnt,
+                                          double *jrec)
 {
-    LegView L;
-    L.t0 = 0.0;
-    L.h = __longlong_as_double(0x7ff8000000000000ll);
-    L.r64 = nullptr;
-    L.r32 = nullptr;
-    L.stride = 0;
-    if (nt) {
-        L.stride = nt->nb * 6;
-        L.t0 = __ldg(nt->t0 + kg);
-        L.h = __ldg(nt->h + kg);
-        L.r64 = nt->row64 + (size_t)kg * 8 * L.stride;
-        L.r32 = nt->row32 + (size_t)kg * 8 * L.stride;
+    if (S.have_a0) return KETE_BODY_OK;
+    const double zero[3] = {0.0, 0.0, 0.0};
+    int st = accel<MODE, JAC>(E, F, t, 0.0, r64, r32, S.close, x, v, S.a0, S.as0, S.enc, zero,
+                                 true, jrec, S.ng, nullptr, &S.ng_chi);
+    cnt.evals++;
+    if (r64) cnt.node_evals++;
+    if (st != KETE_BODY_OK) return st;
+    S.bound = forward ? __longlong_as_double(0x7ff0000000000000ll)
+                      : __longlong_as_double(0xfff0000000000000ll);
+    if (S.enc.m >= 0) {
+        const double k = floor((t - E.t_start) * E.inv_seg);
+        double b = forward ? E.t_start + (k + 1.0) * E.seg_len : E.t_start + k * E.seg_len;
+        if (!forward && b == t) b = E.t_start + (k - 1.0) * E.seg_len;
+        S.bound = b;
     }
-    return L;
-}
-
-// Start a step attempt of (x, v, t) toward `target` (t != target): the
-// acceleration at the step start if it is not known yet (kept across a
-// rejection), the step size and its node rows, the corrector state A.
-// Returns a KETE_BODY_* status.  JAC: as attempt_sweep (jrec[0..5] at t).
-template <int MODE, bool JAC = false, int G = 1>
-__device__ __forceinline__ int step_begin(const EphemDev &E, const ForceDev &F, const LegView &L,
-                                          const double x[3], const double v[3], double t,
-                                          double dt, double target, StepState &S, Attempt &A,
-                                          Cnt &cnt, double *jrec = nullptr)
-{
-    // rows of node 0 serve a0 whenever the step starts at the leg start
-    const bool at_start = L.r64 && (t == L.t0) && isfinite(L.h);
-    if (!S.have_a0) {
-        const double zero[3] = {0.0, 0.0, 0.0};
-        int st = accel<MODE, JAC, G>(E, F, t, 0.0, at_start ? L.r64 : nullptr,
-                                     at_start ? L.r32 : nullptr, S.close, x, v, S.a0, S.as0,
-                                     S.enc, zero, true, jrec, S.ng, nullptr, &S.ng_chi);
-        cnt.evals++;
-        if (at_start) cnt.node_evals++;
-        if (st != KETE_BODY_OK) return st;
-        // during an encounter no step straddles a boundary of the planet polynomials
-        S.t_stop = target;
-        if (S.enc.m >= 0) {
-            const double k = floor((t - E.t_start) * E.inv_seg);
-            double b = (target > t) ? E.t_start + (k + 1.0) * E.seg_len : E.t_start + k * E.seg_len;
-            if (target < t && b == t) b = E.t_start + (k - 1.0) * E.seg_len;
-            if ((target > t && b < target) || (target < t && b > target)) S.t_stop = b;
-        }
-        S.have_a0 = true;
-    }
-    const double remaining = S.t_stop - t;
-    const bool clamped = fabs(dt) >= fabs(remaining);
-    // the step is the exact difference of the representable epochs it joins
-    const double t_new = clamped ? S.t_stop : t + dt;
-    const double h = t_new - t;
-    if (h == 0.0) return KETE_BODY_STEP_CAP;   // step below the epoch resolution
-    LegRows rows = {nullptr, nullptr, L.stride};
-    if (at_start && h == L.h) {
-        rows.r64 = L.r64;
-        rows.r32 = L.r32;
-    }
-    attempt_begin(A, h, t_new, rows);
+    S.have_a0 = true;
     return KETE_BODY_OK;
 }
 
+// Begin the attempt of size dt, clamped at `target` (or the encounter's
+// boundary when that is nearer), planets per thread.
+__device__ __forceinline__ int step_aim(double t, double dt, double target, const StepState &S,
+                                        Attempt &A)
+{
+    double t_stop = target;
+    if ((target > t && S.bound < target) || (target < t && S.bound > target)) t_stop = S.bound;
+    const bool clamped = fabs(dt) >= fabs(t_stop - t);
+    // the step is the exact difference of the representable epochs it joins
+    const double t_new = clamped ? t_stop : t + dt;
+    const double h = t_new - t;
+    if (h == 0.0) return KETE_BODY_STEP_CAP;   // step below the epoch resolution
+    attempt_begin(A, h, t_new, StepRows{nullptr, nullptr, 0});
+    return KETE_BODY_OK;
+}
+
+// Start a step attempt of (x, v, t) toward `target` (t != target): the
+// acceleration at the step start, the step size, the corrector state A.
+// Returns a KETE_BODY_* status.  JAC: as attempt_sweep (jrec[0..5] at t).
+template <int MODE, bool JAC = false>
+__device__ __forceinline__ int step_begin(const EphemDev &E, const ForceDev &F, const double x[3],
+                                          const double v[3], double t, double dt, double target,
+                                          StepState &S, Attempt &A, Cnt &cnt,
+                                          double *jrec = nullptr)
+{
+    const int st = step_start<MODE, JAC>(E, F, nullptr, nullptr, x, v, t, target > t, S, cnt,
+                                            jrec);
+    return st != KETE_BODY_OK ? st : step_aim(t, dt, target, S, A);
+}
+
+// Index of the first grid point at or past t in the grid's direction.
+__device__ __forceinline__ int grid_locate(const GridDev &Q, double t)
+{
+    int lo = 0, hi = Q.J;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        const double g = __ldg(Q.g + mid);
+        if (Q.dir > 0 ? g >= t : g <= t) hi = mid;
+        else lo = mid + 1;
+    }
+    return lo;
+}
+
+// As step_begin for a body that follows the grid Q (j: the grid point it
+// stands on or the next one): from a grid point the longest tabulated step
+// that does not exceed the proposed dt, its planets read from the rows; off the
+// grid a step up to the next grid point, and with a proposal below one unit a
+// step of dt, the planets summed per thread.  jn: the first grid point at or
+// past the step's end.
+template <int MODE>
+__device__ __forceinline__ int step_begin_grid(const EphemDev &E, const ForceDev &F,
+                                               const GridDev &Q, int j, int &jn,
+                                               const double x[3], const double v[3], double t,
+                                               double dt, StepState &S, Attempt &A, Cnt &cnt)
+{
+    const bool on = t == __ldg(Q.g + j);
+    const int stride = Q.nb * 6;
+    const size_t cell = (size_t)8 * stride;
+    const bool row0 = on && j < Q.J && __ldg(Q.ok + (size_t)j * Q.n_len);
+    const size_t at0 = (size_t)j * Q.n_len * cell;
+    const int st = step_start<MODE, false>(E, F, row0 ? Q.row64 + at0 : nullptr,
+                                              row0 ? Q.row32 + at0 : nullptr, x, v, t, Q.dir > 0, S,
+                                              cnt, nullptr);
+    if (st != KETE_BODY_OK) return st;
+    if (on) {
+        const double units = fabs(dt) * Q.inv_unit * (1.0 + 1e-12);
+        const int most = units < (double)(Q.J - j) ? (int)units : Q.J - j;
+        for (int q = Q.n_len - 1; q >= 0; q--) {
+            const int len = Q.len[q];
+            if (len > most || !__ldg(Q.ok + (size_t)j * Q.n_len + q)) continue;
+            const double t_new = __ldg(Q.g + j + len);
+            if (Q.dir > 0 ? t_new > S.bound : t_new < S.bound) continue;
+            const size_t at = ((size_t)j * Q.n_len + q) * cell;
+            attempt_begin(A, t_new - t, t_new, StepRows{Q.row64 + at, Q.row32 + at, stride});
+            jn = j + len;
+            return KETE_BODY_OK;
+        }
+    }
+    jn = on ? j + 1 : j;
+    if (fabs(dt) * Q.inv_unit >= 1.0) return step_aim(t, dt, __ldg(Q.g + jn), S, A);
+    const int st2 = step_aim(t, dt, __ldg(Q.g + Q.J), S, A);
+    while (jn < Q.J && (Q.dir > 0 ? __ldg(Q.g + jn) < A.t_new : __ldg(Q.g + jn) > A.t_new)) jn++;
+    return st2;
+}
+
+// The body's state at epoch ts inside the attempt A from (t, x0, v0, a0): the
+// collocation polynomial of the corrector (the node predictor's sums at
+// s = (ts - t) / h instead of a node).  The polynomial interpolates the
+// acceleration through the 8 nodes; with b6 / |a| held near 1e-9 by the step
+// control its interpolation error, times h^2 |a|, stays orders of magnitude
+// below the rounding of the position.
+__device__ __forceinline__ void attempt_dense(const Attempt &A, double t, const double x0[3],
+                                              const double v0[3], const double a0[3], double ts,
+                                              double xs[3], double vs[3])
+{
+    const double sh = ts - t;
+    const double s = sh / A.h;
+    double wx[7], wv[7], sp = s;
+    constexpr double cx[7] = {1.0 / 6.0,  1.0 / 12.0, 1.0 / 20.0, 1.0 / 30.0,
+                              1.0 / 42.0, 1.0 / 56.0, 1.0 / 72.0};
+    constexpr double cv[7] = {1.0 / 2.0, 1.0 / 3.0, 1.0 / 4.0, 1.0 / 5.0,
+                              1.0 / 6.0, 1.0 / 7.0, 1.0 / 8.0};
+#pragma unroll
+    for (int k = 0; k < 7; k++) {
+        wx[k] = sp * cx[k];
+        wv[k] = sp * cv[k];
+        sp *= s;
+    }
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        double px = A.b[6][i] * wx[6], pv = A.b[6][i] * wv[6];
+#pragma unroll
+        for (int k = 5; k >= 0; k--) {
+            px = fma(A.b[k][i], wx[k], px);
+            pv = fma(A.b[k][i], wv[k], pv);
+        }
+        px = fma(a0[i], 0.5, px);
+        xs[i] = x0[i] + fma(sh * sh, px, sh * v0[i]);
+        vs[i] = fma(sh, pv + a0[i], v0[i]);
+    }
+}
+
+// IAS15's step factor (eps / err)^(1/7), at most 1 / safety (also for an err
+// of zero or none).  The power in FP32: a step proposal needs no more than its
+// 1e-7, and the FP64 pow cost as much issue time as a force evaluation.
+__device__ __forceinline__ double step_factor(const ForceDev &F, double err)
+{
+    const double most = 1.0 / F.safety;
+    if (!(isfinite(err) && err > 1e-37)) return most;
+    const float e = (float)fmin(err, 1e37);
+    return fmin((double)exp2f((F.log2_eps - log2f(e)) * (1.0f / 7.0f)), most);
+}
+
 // End a step attempt whose corrector is done: IAS15 step control.  Accepted:
-// the state advances and dt holds the next proposal.  Rejected: dt shrinks and
-// a0 is kept.  Returns a KETE_BODY_* status.
+// (x1, v1) is the state at the step end and dt holds the next proposal.
+// Rejected: dt shrinks and a0 is kept.  Returns a KETE_BODY_* status.
+template <int MODE>
+__device__ __forceinline__ int step_control(const ForceDev &F, const Attempt &A, const double x[3],
+                                            const double v[3], double &dt, const StepState &S,
+                                            Cnt &cnt, double x1[3], double v1[3], bool &accepted)
+{
+    double err;
+    accepted = false;
+    int st = attempt_end<MODE>(A, x, v, S.a0, x1, v1, err);
+    if (st != KETE_BODY_OK) return st;
+    const double h = A.h;
+    const double factor = step_factor(F, err);
+    dt = factor * h;
+    if (factor < F.safety) {   // reject: retry from the same a0
+        cnt.rejected++;
+        return KETE_BODY_OK;
+    }
+    accepted = true;
+    cnt.steps++;
+    return KETE_BODY_OK;
+}
+
+// step_control, and the state advanced when the step was accepted
 template <int MODE>
 __device__ __forceinline__ int step_end(const ForceDev &F, const Attempt &A, double x[3],
                                         double v[3], double &t, double &dt, StepState &S, Cnt &cnt)
 {
-    double x1[3], v1[3], err;
-    int st = attempt_end<MODE>(A, x, v, S.a0, x1, v1, err);
-    if (st != KETE_BODY_OK) return st;
-    const double h = A.h;
-    double dt_new;
-    if (isfinite(err) && err >= 2.2250738585072014e-308)
-        dt_new = pow(F.eps / err, 1.0 / 7.0) * h;
-    else
-        dt_new = h / F.safety;
-    if (fabs(dt_new / h) < F.safety) {   // reject: retry from the same a0
-        dt = dt_new;
-        cnt.rejected++;
-        return KETE_BODY_OK;
-    }
-    if (fabs(dt_new / h) > 1.0 / F.safety) dt_new = h / F.safety;
-    dt = dt_new;
+    double x1[3], v1[3];
+    bool accepted;
+    const int st = step_control<MODE>(F, A, x, v, dt, S, cnt, x1, v1, accepted);
+    if (st != KETE_BODY_OK || !accepted) return st;
 #pragma unroll
     for (int i = 0; i < 3; i++) {
         x[i] = x1[i];
@@ -428,7 +528,6 @@ __device__ __forceinline__ int step_end(const ForceDev &F, const Attempt &A, dou
     }
     t = A.t_new;
     S.have_a0 = false;
-    cnt.steps++;
     return KETE_BODY_OK;
 }
 
@@ -436,18 +535,17 @@ __device__ __forceinline__ int step_end(const ForceDev &F, const Attempt &A, dou
 // step_begin, corrector sweeps until done, step_end.
 // JAC: da/dx at the 8 nodes of the attempt go to jrec[6n..6n+5]; after an
 // accepted step they describe that step.
-template <int MODE, bool JAC = false, int G = 1>
-__device__ __forceinline__ int step_once(const EphemDev &E, const ForceDev &F, const LegView &L,
-                                         double x[3], double v[3], double &t, double &dt,
-                                         double target, StepState &S, Cnt &cnt,
-                                         double *jrec = nullptr)
+template <int MODE, bool JAC = false>
+__device__ __forceinline__ int step_once(const EphemDev &E, const ForceDev &F, double x[3],
+                                         double v[3], double &t, double &dt, double target,
+                                         StepState &S, Cnt &cnt, double *jrec = nullptr)
 {
     Attempt A;
-    int st = step_begin<MODE, JAC, G>(E, F, L, x, v, t, dt, target, S, A, cnt, jrec);
+    int st = step_begin<MODE, JAC>(E, F, x, v, t, dt, target, S, A, cnt, jrec);
     if (st != KETE_BODY_OK) return st;
     for (;;) {
         bool done = false;
-        st = attempt_sweep<MODE, JAC, G>(E, F, t, x, v, S.a0, S.as0, S.close, S.enc, A, done, cnt,
+        st = attempt_sweep<MODE, JAC>(E, F, t, x, v, S.a0, S.as0, S.close, S.enc, A, done, cnt,
                                          jrec, S.ng, &S.ng_chi);
         if (st != KETE_BODY_OK) return st;
         if (done) break;
@@ -462,14 +560,10 @@ __device__ __forceinline__ void aim_step(const ForceDev &F, double t, double tar
     if (dt == 0.0 || ((dt > 0.0) != (dir > 0.0))) dt = dir * fabs(dt == 0.0 ? F.dt_init : dt);
 }
 
-// warp sums of the lanes' counters into ctr; with G lanes per body only the
-// rank-0 lane of a group counts
-template <int G = 1>
+// warp sums of the lanes' counters into ctr
 __device__ __forceinline__ void flush_counters(const Cnt &c, DevCounters *ctr)
 {
-    const unsigned long long w = (LaneGroup<G>::rank() == 0) ? 1ull : 0ull;
-    unsigned long long s = w * c.steps, r = w * c.rejected, e = w * c.evals, it = w * c.iters,
-                       ne = w * c.node_evals;
+    unsigned long long s = c.steps, r = c.rejected, e = c.evals, it = c.iters, ne = c.node_evals;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         s += __shfl_xor_sync(0xffffffffu, s, o);
