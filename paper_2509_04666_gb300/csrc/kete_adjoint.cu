@@ -649,7 +649,7 @@ k_adj_forward(EphemDev E, ForceDev F, AdjBuffers B, AdjProblem P, int64_t i0, in
                         if (done) break;
                     }
                     if (status == KETE_BODY_OK)
-                        status = step_end<KETE_FP64>(F, A, x, v, t, dt, S, cnt);
+                        status = step_end<KETE_FP64, true>(F, A, x, v, t, dt, S, cnt);
                     if (status == KETE_BODY_OK && t != t_prev)
                         status = record_extra(E, F, t_prev, x0, v0, S.a0, A, S.ng,
                                               recx + (size_t)slot * kAdjRecX);

@@ -412,7 +412,7 @@ __device__ __forceinline__ int accel_fp64(const EphemDev &E, const ForceDev &F, 
                                           const double x[3], const double v[3], double a[3],
                                           Encounter &enc, const double dx[3], bool detect,
                                           double *J = nullptr, const kete_nongrav *ng = nullptr,
-                                          double *ng_chi = nullptr)
+                                          double *ng_chi = nullptr, double *helio = nullptr)
 {
     Seg g = {0, 0.0};
     a[0] = a[1] = a[2] = 0.0;
@@ -462,6 +462,13 @@ __device__ __forceinline__ int accel_fp64(const EphemDev &E, const ForceDev &F, 
                 enc.m = m;
                 enc.d0[0] = r[0]; enc.d0[1] = r[1]; enc.d0[2] = r[2];
             }
+            if (m == 0 && helio) {   // (without a GR term the Sun's own velocity is left out)
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    helio[c] = r[c];
+                    helio[3 + c] = v[c] - st[3 + c];
+                }
+            }
         } else if (m == enc.m) {
             double dp[3];
             cheb_delta64(E, m, enc.t0, off, dp);
@@ -510,7 +517,8 @@ __device__ __forceinline__ int accel_mixed(const EphemDev &E, const ForceDev &F,
                                            const double x[3], const double v[3], double a[3],
                                            double as[3], Encounter &enc, const double dx[3],
                                            bool detect, const kete_nongrav *ng = nullptr,
-                                           const float *vf_in = nullptr, double *ng_chi = nullptr)
+                                           const float *vf_in = nullptr, double *ng_chi = nullptr,
+                                           double *helio = nullptr)
 {
     Seg g = {0, 0.0};
     as[0] = as[1] = as[2] = 0.0;
@@ -543,6 +551,13 @@ __device__ __forceinline__ int accel_mixed(const EphemDev &E, const ForceDev &F,
     }
     const double d[3] = {x[0] - sun[0], x[1] - sun[1], x[2] - sun[2]};
     const float df[3] = {(float)d[0], (float)d[1], (float)d[2]};
+    if (helio) {
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            helio[c] = d[c];
+            helio[3 + c] = v[c] - (double)sunv[c];
+        }
+    }
     // the body's velocity enters only FP32 terms: taken in FP32 when the
     // caller has it (vf_in), else rounded here
     float vf[3];

@@ -37,7 +37,8 @@ struct ForceDev {
     // 4 mu / c^2 and -2 x the pole
     double gm4[KETE_MAX_BODIES], grk[KETE_MAX_BODIES], gr4k[KETE_MAX_BODIES];
     double pole_m2[KETE_MAX_BODIES][3];
-    double eps, eps_pc, safety, dt_init;
+    double eps, safety, dt_init;
+    double eps_pc;           // the caller's threshold as the analytic start needs it (make_force)
     int32_t max_iter;
     float log2_eps;
     int64_t max_steps;

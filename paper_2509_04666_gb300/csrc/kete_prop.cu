@@ -65,9 +65,8 @@ __device__ __forceinline__ void write_stop(double *__restrict__ out,
 // whatever its active lanes, so the work between attempts (step control, the
 // stops inside the step, the next body, the acceleration at the next step's
 // start: about a third of a sweep) waits until kSyncLanes lanes have reached
-// it or none is left in an attempt; nearly all attempts take four sweeps, and
-// lanes that have met there stay together (757,000 bodies over 60 days: 228 ms
-// without waiting, 161 for 8 lanes, 125 for 16, 111 for 24 and for 30).
+// it or none is left in an attempt (400,000 main-belt bodies over 60 days: 40.8
+// ms for 8 lanes, 39.1 for 16, 40.2 for 24, 40.3 for 32).
 //   refill = 0 (static): lane j of the grid takes body j and then idles;
 //   refill = 1 (work stealing, persistent grid): a lane whose body is done
 //   takes the next one from an atomic counter (warp-aggregated), so a body
@@ -83,7 +82,7 @@ __device__ __forceinline__ void write_stop(double *__restrict__ out,
 // per-thread planet sums would be paid by the whole warp.
 // NG: bodies may carry non-gravitational terms (F.nongrav); the instantiation
 // without them has those branches compiled out.
-constexpr int kSyncLanes = 28;
+constexpr int kSyncLanes = 16;
 template <int MODE, bool NG, bool V32 = false>
 __global__ void __launch_bounds__(128, KETE_PROP_MIN_BLOCKS)
 k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ stops,
@@ -258,8 +257,11 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                 }
             }
         }
-        // one corrector sweep for every lane inside an attempt
-        if (phase == SWEEP) {
+        // the lanes that have just begun a step and the others sweep together (they
+        // left the branches above apart: 757,000 bodies over 60 days 108 ms
+        // without this, 85 with it)
+        __syncwarp(FULL);
+        if (phase == SWEEP) {   // one corrector sweep
             bool done = false;
             status = attempt_sweep<MODE, false, V32>(E, F, t, x, v, S.a0, S.as0, S.close, S.enc, A,
                                                      done, cnt, nullptr, S.ng, &S.ng_chi);

@@ -241,6 +241,9 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
         ri[k] = node > k ? g_rt.rinv[node][k] : 0.0;
     }
     const int max_sweeps = F.max_iter + 4;
+    // the change of F between sweeps at the nodes, relative to |a|: one sweep more
+    // contracts what is left by ~1e-3, below the rounding of the positions
+    const float tol = (float)(0.3 * F.eps_pc);
     for (unsigned long long item = blockIdx.x; item < n_items; item += gridDim.x) {
         const int64_t i = q.list ? (int64_t)q.list[item] : (int64_t)item;
         // own coordinate of the step-start state
@@ -253,6 +256,7 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
         long long attempts = 0;
         bool careful = false, have_a0 = false;
         double a0 = 0.0, bound = inf;
+        double d1 = 0.0, d2 = 0.0, d3 = 0.0;   // derivatives of a at the step start
         int enc_m = -1, enc_slot = -1;
         double d0[3] = {0.0, 0.0, 0.0};
         while (k < n_stops && status == KETE_BODY_OK) {
@@ -339,6 +343,18 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
                 const int s2 = own_terms(node == 0, xs, vs, own);
                 const double f = node_force(W, M, xs, vs, zero, -1, d0, r, own);
                 a0 = __shfl_sync(kFull, f, r);
+                {   // the corrector's start (two_body_derivs), from the Sun in lane 0
+                    double hr[3], hw[3], e1[3], e2[3], e3[3];
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+                        hr[c] = xs[c] - __shfl_sync(kFull, M.p[0][c], 0);
+                        hw[c] = vs[c] - __shfl_sync(kFull, M.w[c], 0);
+                    }
+                    two_body_derivs(E.gm[0], hr, hw, e1, e2, e3);
+                    d1 = rc == 0 ? e1[0] : rc == 1 ? e1[1] : e1[2];
+                    d2 = rc == 0 ? e2[0] : rc == 1 ? e2[1] : e2[2];
+                    d3 = rc == 0 ? e3[0] : rc == 1 ? e3[1] : e3[2];
+                }
                 if (NG && ng) st = __shfl_sync(kFull, s2, 3);
                 cnt.evals++;
 #pragma unroll
@@ -393,7 +409,16 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
                 double Fo = a0;
                 float pc_prev = 0.0f;
 #pragma unroll
-                for (int m = 0; m < 7; m++) g[m] = 0.0;
+                for (int m = 3; m < 7; m++) g[m] = 0.0;
+                {   // as attempt_begin
+                    const double h1 = g_rt.h[1], h2 = g_rt.h[2];
+                    const double b0 = h * d1, b1 = 0.5 * h * h * d2, b2 = h * h * h * (1.0 / 6.0) * d3;
+                    g[2] = b2;
+                    g[1] = fma(h1 + h2, b2, b1);
+                    g[0] = fma(h1, g[1], fma(-h1 * h2, b2, b0));
+                    // what the start predicts at the node
+                    Fo = fma(fma(fma(d3, sh * (1.0 / 3.0), d2), 0.5 * sh, d1), sh, a0);
+                }
                 for (int it = 1;; it++) {
                     double px = g[6] * wx[6], pv = g[6] * wv[6];
 #pragma unroll
@@ -438,7 +463,7 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
                         st = KETE_BODY_NONFINITE;
                         break;
                     }
-                    if (pc < (float)F.eps_pc || (it >= 3 && pc >= pc_prev) || it >= max_sweeps) break;
+                    if (pc < tol || (it >= 3 && pc >= pc_prev) || it >= max_sweeps) break;
                     pc_prev = pc;
                 }
                 b6 = fabs(g[6]);
