@@ -34,7 +34,7 @@ enum Slot {
     S_ORDER_SCAN, S_ORDER_N, S_ADJ_TEND, S_LEG_OUT,
     S_EXT_START, S_EXT_EX, S_EXT_TMP, S_EXT_FIRST, S_EXT_SUB, S_EXT_PARENT, S_EXT_CNT,
     S_EXT_OFF, S_EXT_CUR, S_EXT_GROUP, S_EXT_KEEP, S_EXT_KCNT, S_EXT_KOFF, S_ADJ_PHI, S_ADJ_RECX,
-    S_PRE_KEEP, S_PRE_N, S_ADJ_RICH,
+    S_PRE_KEEP, S_PRE_N, S_ADJ_RICH, S_ADJ_PLANETS,
     S_NSLOTS
 };
 
@@ -1483,6 +1483,8 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
             GET(S_ADJ_RECX, (size_t)chunk * cap * kAdjRecX, B.recx);
             GET(S_ADJ_RICH, chunk, B.rich);
         }
+        GET(S_ADJ_PLANETS, (size_t)adjoint_forward_lanes(chunk, full) * 7 * ctx->E.n_bodies * 6,
+            B.planets);
         unsigned long long *next = nullptr;
         GET(S_NEXTBODY, 1, next);
         int launches = 0;

@@ -13,7 +13,7 @@
 //                   Gauss-Radau nodes, taken from the force evaluations the
 //                   step already makes.  The state at each batch midpoint is
 //                   kept for the sky projection.
-//   k_adj_observe   one warp per body, one lane per observation: prediction,
+//   k_adj_observe   one thread per observation: prediction,
 //                   residual, loss term and dL/dy(t_ref) through RA/Dec, the
 //                   light-time fixed point (implicit derivative) and the
 //                   universal-variable two-body map (forward-mode dual numbers
@@ -531,22 +531,30 @@ __device__ __forceinline__ void walk_next_ckpt(StopWalk &w, double epoch0, doubl
     w.ckpt_ok = w.tc < w.t_last;
 }
 
-// One lane per body at a time, one step attempt per loop iteration (lanes of a
-// warp stay in step while their bodies sit at different stops).  refill = 1:
-// persistent grid, a lane whose body is done takes the next one from *next.
+// One lane per body at a time; a pass of the loop is one corrector sweep, and
+// the work between attempts waits until kAdjSyncLanes lanes have reached it or
+// none is left in an attempt (as k_propagate; FP64 issue bounds this kernel, and
+// an FP64 warp instruction costs the same whatever its active lanes).  The
+// planets of an attempt's nodes are summed in its first sweep and read back in
+// the others (B.planets; 430 of a node's 900 FP64 instructions, 2.9 sweeps).
+// Neither changes any arithmetic.  Persistent grid: a lane whose body is done
+// takes the next one from *next.
 // RICH: a body with non-gravitational terms has them in its force, and each
 // of its records gets the full model's Jacobian (B.recx) besides the
 // Newtonian da/dx; a body whose terms are all zero keeps the Newtonian
 // records (B.rich[i] tells which).
+constexpr int kAdjSyncLanes = 16;
 template <bool RICH>
 __global__ void __launch_bounds__(128)
 k_adj_forward(EphemDev E, ForceDev F, AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc,
-              unsigned long long *__restrict__ next, int refill, const int32_t *__restrict__ order)
+              unsigned long long *__restrict__ next, const int32_t *__restrict__ order)
 {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
+    const int64_t pstride = (int64_t)gridDim.x * blockDim.x;
+    double *planets = B.planets + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     Cnt cnt = {0, 0, 0, 0, 0};
-    int64_t i = -1;   // current body (chunk index); -1: none; nc: no work left
+    int64_t i = 0;   // current body (chunk index)
     double x[3], v[3], t = 0.0, dt = 0.0, epoch0 = 0.0, ts = 0.0;
     bool mid = false, capped = false;
     int status = KETE_BODY_OK, count = 0;
@@ -557,166 +565,174 @@ k_adj_forward(EphemDev E, ForceDev F, AdjBuffers B, AdjProblem P, int64_t i0, in
     S.have_a0 = false;
     S.ng = nullptr;   // set per body on the full-model path
     S.ng_chi = 0.0;
+    Attempt A;
     double *rec = nullptr, *recx = nullptr;   // recx: null for a body without terms
-    bool first = true;
+    enum { TAKE, BOUNDARY, SWEEP, SWEPT, DRAINED };
+    int phase = TAKE;
     for (;;) {
-        const bool need = (i < 0);
-        const unsigned m = __ballot_sync(FULL, need);
-        if (m) {
-            unsigned long long base = 0;
-            const int leader = __ffs(m) - 1;
-            if (refill) {
-                if (lane == leader) base = atomicAdd(next, (unsigned long long)__popc(m));
-                base = __shfl_sync(FULL, base, leader);
-            }
-            if (need) {
-                unsigned long long mine = base + __popc(m & ((1u << lane) - 1u));
-                if (!refill)
-                    mine = first ? (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x
-                                 : (unsigned long long)nc;
-                if (mine < (unsigned long long)nc) {
-                    i = order ? (int64_t)order[mine] : (int64_t)mine;
-                    const int64_t gi = i0 + i;
-                    o = P.obs + gi * P.m;
-                    bool fin = true;
-#pragma unroll
-                    for (int c = 0; c < 3; c++) {
-                        x[c] = P.states[c * P.n + gi];
-                        v[c] = P.states[(3 + c) * P.n + gi];
-                        fin = fin && isfinite(x[c]) && isfinite(v[c]);
-                    }
-                    epoch0 = P.epochs[gi];
-                    t = epoch0;
-                    dt = 0.0;
-                    status = (fin && isfinite(epoch0)) ? KETE_BODY_OK : KETE_BODY_NONFINITE;
-                    W.mi = obs_count(o, P.m);
-                    for (int j = 1; j < W.mi; j++)
-                        if (o[j].epoch < o[j - 1].epoch) {
-                            atomicOr(&P.ctr->error_flags, 1 << 6);
-                            status = KETE_BODY_NONFINITE;
-                        }
-                    // batches and the last midpoint (the checkpoint grid ends there)
-                    W.nb = 0;
-                    W.t_last = epoch0;
-                    for (int j0 = 0; j0 < W.mi; W.nb++) j0 = next_batch(o, W.mi, j0, P.span, W.t_last);
-                    W.kb = 0;
-                    W.j1 = (W.mi > 0) ? next_batch(o, W.mi, 0, P.span, W.tref) : 0;
-                    W.kc = 1;
-                    W.tc = epoch0 + P.ckpt;
-                    W.ckpt_ok = P.ckpt > 0.0 && W.tc < W.t_last;
-                    rec = B.rec + (size_t)i * B.cap * kAdjRec;
-                    if (RICH) {
-                        const kete_nongrav *p = F.nongrav ? F.nongrav + gi : nullptr;
-                        const bool terms = p && (p->a1 != 0.0 || p->a2 != 0.0 ||
-                                                 p->a3 != 0.0 || p->beta != 0.0);
-                        recx = terms ? B.recx + (size_t)i * B.cap * kAdjRecX : nullptr;
-                        S.ng = terms ? p : nullptr;
-                        S.ng_chi = 0.0;
-                    }
-                    count = 0;
-                    capped = false;
-                    attempts = 0;
-                    S.have_a0 = false;
-                    if (W.kb < W.nb) {
-                        ts = walk_target(W, mid);
-                        aim_step(F, t, ts, dt);
-                    }
-                } else {
-                    i = nc;
-                }
-            }
-        }
-        first = false;
-        const bool active = (i >= 0 && i < nc);
-        if (!__any_sync(FULL, active)) break;
-        if (!active) continue;
-        if (status == KETE_BODY_OK && W.kb < W.nb && t != ts) {
-            if (++attempts > F.max_steps) {
-                status = KETE_BODY_STEP_CAP;
-            } else {
+        const unsigned sweeping = __ballot_sync(FULL, phase == SWEEP);
+        const unsigned waiting = __ballot_sync(FULL, phase != SWEEP && phase != DRAINED);
+        if (!(sweeping | waiting)) break;
+        if (waiting && (!sweeping || __popc(waiting) >= kAdjSyncLanes)) {
+            if (phase == SWEPT) {
+                phase = BOUNDARY;
                 const int slot = count < B.cap - 1 ? count : B.cap - 2;
-                double *r = rec + (size_t)slot * kAdjRec;
                 const double t_prev = t;
-                if (RICH && recx) {   // the accepted attempt's coefficients give the node states
-                    const double x0[3] = {x[0], x[1], x[2]}, v0[3] = {v[0], v[1], v[2]};
-                    Attempt A;
-                    status = step_begin<KETE_FP64, true>(E, F, x, v, t, dt, ts, S, A, cnt, r + 2);
-                    while (status == KETE_BODY_OK) {
-                        bool done = false;
-                        status = attempt_sweep<KETE_FP64, true>(E, F, t, x, v, S.a0, S.as0,
-                                                                S.close, S.enc, A, done, cnt,
-                                                                r + 2, S.ng, &S.ng_chi);
-                        if (done) break;
-                    }
-                    if (status == KETE_BODY_OK)
-                        status = step_end<KETE_FP64, true>(F, A, x, v, t, dt, S, cnt);
-                    if (status == KETE_BODY_OK && t != t_prev)
-                        status = record_extra(E, F, t_prev, x0, v0, S.a0, A, S.ng,
-                                              recx + (size_t)slot * kAdjRecX);
-                } else {
-                    status = step_once<KETE_FP64, true>(E, F, x, v, t, dt, ts, S, cnt, r + 2);
-                }
+                const double x0[3] = {x[0], x[1], x[2]}, v0[3] = {v[0], v[1], v[2]};
+                if (status == KETE_BODY_OK)
+                    status = step_end<KETE_FP64, true>(F, A, x, v, t, dt, S, cnt);
+                if (RICH && recx && status == KETE_BODY_OK && t != t_prev)
+                    // the accepted attempt's coefficients give the node states
+                    status = record_extra(E, F, t_prev, x0, v0, S.a0, A, S.ng,
+                                          recx + (size_t)slot * kAdjRecX);
                 if (status == KETE_BODY_OK && t != t_prev) {
+                    double *r = rec + (size_t)slot * kAdjRec;
                     r[0] = t_prev;
                     r[1] = t;
                     if (count < B.cap - 1) count++;
                     else capped = true;
                 }
             }
-            if (status == KETE_BODY_OK && t != ts) continue;
-        }
-        // at the stop ts (or failed): bookkeeping, then the next stop
-        if (status == KETE_BODY_OK && W.kb < W.nb) {
-            if (mid) {
-                double *y = B.yref + ((size_t)i * P.m + W.kb) * 6;
+            for (;;) {
+                const bool need = phase == TAKE;
+                const unsigned m = __ballot_sync(FULL, need);
+                if (m) {
+                    unsigned long long base = 0;
+                    const int leader = __ffs(m) - 1;
+                    if (lane == leader) base = atomicAdd(next, (unsigned long long)__popc(m));
+                    base = __shfl_sync(FULL, base, leader);
+                    if (need) {
+                        const unsigned long long mine = base + __popc(m & ((1u << lane) - 1u));
+                        if (mine < (unsigned long long)nc) {
+                            i = order ? (int64_t)order[mine] : (int64_t)mine;
+                            const int64_t gi = i0 + i;
+                            o = P.obs + gi * P.m;
+                            bool fin = true;
 #pragma unroll
-                for (int c = 0; c < 3; c++) {
-                    y[c] = x[c];
-                    y[3 + c] = v[c];
+                            for (int c = 0; c < 3; c++) {
+                                x[c] = P.states[c * P.n + gi];
+                                v[c] = P.states[(3 + c) * P.n + gi];
+                                fin = fin && isfinite(x[c]) && isfinite(v[c]);
+                            }
+                            epoch0 = P.epochs[gi];
+                            t = epoch0;
+                            dt = 0.0;
+                            status = (fin && isfinite(epoch0)) ? KETE_BODY_OK : KETE_BODY_NONFINITE;
+                            W.mi = obs_count(o, P.m);
+                            for (int j = 1; j < W.mi; j++)
+                                if (o[j].epoch < o[j - 1].epoch) {
+                                    atomicOr(&P.ctr->error_flags, 1 << 6);
+                                    status = KETE_BODY_NONFINITE;
+                                }
+                            // batches and the last midpoint (the checkpoint grid ends there)
+                            W.nb = 0;
+                            W.t_last = epoch0;
+                            for (int j0 = 0; j0 < W.mi; W.nb++) j0 = next_batch(o, W.mi, j0, P.span, W.t_last);
+                            W.kb = 0;
+                            W.j1 = (W.mi > 0) ? next_batch(o, W.mi, 0, P.span, W.tref) : 0;
+                            W.kc = 1;
+                            W.tc = epoch0 + P.ckpt;
+                            W.ckpt_ok = P.ckpt > 0.0 && W.tc < W.t_last;
+                            rec = B.rec + (size_t)i * B.cap * kAdjRec;
+                            if (RICH) {
+                                const kete_nongrav *p = F.nongrav ? F.nongrav + gi : nullptr;
+                                const bool terms = p && (p->a1 != 0.0 || p->a2 != 0.0 ||
+                                                         p->a3 != 0.0 || p->beta != 0.0);
+                                recx = terms ? B.recx + (size_t)i * B.cap * kAdjRecX : nullptr;
+                                S.ng = terms ? p : nullptr;
+                                S.ng_chi = 0.0;
+                            }
+                            count = 0;
+                            capped = false;
+                            attempts = 0;
+                            S.have_a0 = false;
+                            if (W.kb < W.nb) {
+                                ts = walk_target(W, mid);
+                                aim_step(F, t, ts, dt);
+                            }
+                            phase = BOUNDARY;
+                        } else {
+                            phase = DRAINED;
+                        }
+                    }
                 }
-                B.bidx[(size_t)i * P.m + W.kb] = count;
-                if (W.ckpt_ok && W.tc == W.tref) walk_next_ckpt(W, epoch0, P.ckpt);   // one stop
-                W.kb++;
-                if (W.kb < W.nb) W.j1 = next_batch(o, W.mi, W.j1, P.span, W.tref);
-            } else if (W.kc >= kAdjMaxCkpt) {   // bounded work per body
-                status = KETE_BODY_STEP_CAP;
-            } else {
-                walk_next_ckpt(W, epoch0, P.ckpt);
-            }
-            if (status == KETE_BODY_OK && W.kb < W.nb) {
-                ts = walk_target(W, mid);
-                aim_step(F, t, ts, dt);
-                S.have_a0 = false;
-                attempts = 0;
-                continue;
-            }
-        }
-        // the body is done
-        if (status == KETE_BODY_OK && !capped) {
-            // terminal record: da/dx at the final state closes the last step
-            double *r = rec + (size_t)count * kAdjRec;
-            double a[3], J[6];
-            Encounter enc;
-            const double zero[3] = {0.0, 0.0, 0.0};
-            status = accel_fp64<true>(E, F, t, 0.0, nullptr, x, v, a, enc, zero, true, J, S.ng,
-                                      &S.ng_chi);
-            cnt.evals++;
-            r[0] = t;
-            r[1] = t;
+                if (phase == BOUNDARY) {
+                    // the stops the body stands at
+                    while (status == KETE_BODY_OK && W.kb < W.nb && t == ts) {
+                        if (mid) {
+                            double *y = B.yref + ((size_t)i * P.m + W.kb) * 6;
 #pragma unroll
-            for (int q = 0; q < 6; q++) r[2 + q] = J[q];
-            if (RICH && recx && status == KETE_BODY_OK) {
-                double *rx = recx + (size_t)count * kAdjRecX;
-                status = extra_jacobian(E, F, t, 0.0, x, v, S.ng, rx, rx + 9);
+                            for (int c = 0; c < 3; c++) {
+                                y[c] = x[c];
+                                y[3 + c] = v[c];
+                            }
+                            B.bidx[(size_t)i * P.m + W.kb] = count;
+                            if (W.ckpt_ok && W.tc == W.tref) walk_next_ckpt(W, epoch0, P.ckpt);   // one stop
+                            W.kb++;
+                            if (W.kb < W.nb) W.j1 = next_batch(o, W.mi, W.j1, P.span, W.tref);
+                        } else if (W.kc >= kAdjMaxCkpt) {   // bounded work per body
+                            status = KETE_BODY_STEP_CAP;
+                        } else {
+                            walk_next_ckpt(W, epoch0, P.ckpt);
+                        }
+                        if (status == KETE_BODY_OK && W.kb < W.nb) {
+                            ts = walk_target(W, mid);
+                            aim_step(F, t, ts, dt);
+                            S.have_a0 = false;
+                            attempts = 0;
+                        }
+                    }
+                    if (status != KETE_BODY_OK || W.kb >= W.nb) {
+                        // the body is done
+                        if (status == KETE_BODY_OK && !capped) {
+                            // terminal record: da/dx at the final state closes the last step
+                            double *r = rec + (size_t)count * kAdjRec;
+                            double a[3], J[6];
+                            Encounter enc;
+                            const double zero[3] = {0.0, 0.0, 0.0};
+                            status = accel_fp64<true>(E, F, t, 0.0, nullptr, x, v, a, enc, zero,
+                                                      true, J, S.ng, &S.ng_chi);
+                            cnt.evals++;
+                            r[0] = t;
+                            r[1] = t;
+#pragma unroll
+                            for (int q = 0; q < 6; q++) r[2 + q] = J[q];
+                            if (RICH && recx && status == KETE_BODY_OK) {
+                                double *rx = recx + (size_t)count * kAdjRecX;
+                                status = extra_jacobian(E, F, t, 0.0, x, v, S.ng, rx, rx + 9);
+                            }
+                            count++;
+                        }
+                        if (status == KETE_BODY_OK && capped) status = KETE_BODY_ADJ_CAP;
+                        B.n_rec[i] = (status == KETE_BODY_OK) ? count : 0;
+                        B.nbat[i] = W.nb;
+                        B.status[i] = status;
+                        if (RICH) B.rich[i] = recx ? 1 : 0;
+                        phase = TAKE;
+                    }
+                }
+                if (!__any_sync(FULL, phase == TAKE)) break;
             }
-            count++;
+            if (phase == BOUNDARY) {
+                if (++attempts > F.max_steps) {
+                    status = KETE_BODY_STEP_CAP;
+                } else {
+                    const int slot = count < B.cap - 1 ? count : B.cap - 2;
+                    status = step_begin<KETE_FP64, true>(E, F, x, v, t, dt, ts, S, A, cnt,
+                                                         rec + (size_t)slot * kAdjRec + 2);
+                    if (status == KETE_BODY_OK) phase = SWEEP;
+                }
+            }
         }
-        if (status == KETE_BODY_OK && capped) status = KETE_BODY_ADJ_CAP;
-        B.n_rec[i] = (status == KETE_BODY_OK) ? count : 0;
-        B.nbat[i] = W.nb;
-        B.status[i] = status;
-        if (RICH) B.rich[i] = recx ? 1 : 0;
-        i = -1;
+        __syncwarp(FULL);   // the lanes that have just begun a step sweep with the others
+        if (phase == SWEEP) {
+            const int slot = count < B.cap - 1 ? count : B.cap - 2;
+            bool done = false;
+            status = attempt_sweep<KETE_FP64, true>(E, F, t, x, v, S.a0, S.as0, S.close, S.enc, A,
+                                                    done, cnt, rec + (size_t)slot * kAdjRec + 2,
+                                                    S.ng, &S.ng_chi, planets, pstride);
+            if (done || status != KETE_BODY_OK) phase = SWEPT;
+        }
     }
     flush_counters(cnt, P.ctr);
 }
@@ -740,18 +756,24 @@ __device__ __forceinline__ double wrap_pi(double a)
     return a;
 }
 
-// warp per body, lane per observation (m <= 32)
+// Thread per observation slot, 128 / m whole bodies to a block of 128 threads:
+// FP64 issue bounds it (5 two-body solves an observation), and a warp per body
+// left 12 of 32 lanes idle at 20 observations (100,000 bodies: 17.0 ms, now
+// 11.5).  w: the body within the block, lane: its observation.
 __global__ void __launch_bounds__(128)
 k_adj_observe(EphemDev E, AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 {
-    __shared__ double sh[4][32][7];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t i = (int64_t)blockIdx.x * 4 + w;
-    if (i >= nc) return;   // whole warp
+    __shared__ double sh[128][7];
+    __shared__ int body_bad[128];
+    const int w = threadIdx.x / P.m, lane = threadIdx.x % P.m;
+    const int64_t i = (int64_t)blockIdx.x * (128 / P.m) + w;
+    body_bad[threadIdx.x] = 0;
+    __syncthreads();
+    const bool here = w < 128 / P.m && i < nc;
     const int64_t gi = i0 + i;
-    const kete_obs *o = P.obs + gi * P.m;
-    const int mi = obs_count(o, P.m);
-    int st = B.status[i];
+    const kete_obs *o = here ? P.obs + gi * P.m : nullptr;
+    const int mi = here ? obs_count(o, P.m) : 0;
+    int st = here ? B.status[i] : KETE_BODY_NONFINITE;
     // this lane's batch
     int kb = -1, j0 = 0, j1 = 0;
     double tref = 0.0;
@@ -873,27 +895,30 @@ k_adj_observe(EphemDev E, AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
             P.pred[(gi * P.m + lane) * 2] = ra;
             P.pred[(gi * P.m + lane) * 2 + 1] = dec;
         }
-    } else if (P.pred && lane < P.m) {
+    } else if (P.pred && here) {
         P.pred[(gi * P.m + lane) * 2] = ra;
         P.pred[(gi * P.m + lane) * 2 + 1] = dec;
     }
-    if (P.jac && lane < P.m && !jac_done) {   // unused slot or failed body: NaN rows
+    if (P.jac && here && !jac_done) {   // unused slot or failed body: NaN rows
         double *jr = P.jac + (gi * P.m + lane) * 12;
         for (int q = 0; q < 12; q++) jr[q] = __longlong_as_double(0x7ff8000000000000ll);
     }
-    const bool any_bad = __any_sync(0xffffffffu, bad);
-    if (P.jac && any_bad && lane < P.m) {   // a failed body has no Jacobian
-        double *jr = P.jac + (gi * P.m + lane) * 12;
-        for (int q = 0; q < 12; q++) jr[q] = __longlong_as_double(0x7ff8000000000000ll);
-    }
-    sh[w][lane][0] = Lj;
+    if (bad) body_bad[w] = 1;
+    sh[threadIdx.x][0] = Lj;
 #pragma unroll
-    for (int c = 0; c < 6; c++) sh[w][lane][1 + c] = gj[c];
-    __syncwarp();
+    for (int c = 0; c < 6; c++) sh[threadIdx.x][1 + c] = gj[c];
+    __syncthreads();
+    if (!here) return;
+    const bool any_bad = body_bad[w] != 0;
+    const double (*mine_sh)[7] = sh + w * P.m;   // this body's observations
+    if (P.jac && any_bad) {   // a failed body has no Jacobian
+        double *jr = P.jac + (gi * P.m + lane) * 12;
+        for (int q = 0; q < 12; q++) jr[q] = __longlong_as_double(0x7ff8000000000000ll);
+    }
     // loss in observation order; gradient jumps summed per batch in order
     if (lane == 0) {
         double L = 0.0;
-        for (int j = 0; j < mi; j++) L += sh[w][j][0];
+        for (int j = 0; j < mi; j++) L += mine_sh[j][0];
         const bool ok = (st == KETE_BODY_OK || st == KETE_BODY_ADJ_CAP) && !any_bad;
         if (any_bad && st == KETE_BODY_OK) st = KETE_BODY_KEPLER_CAP;
         if (P.loss) P.loss[gi] = ok ? L : __longlong_as_double(0x7ff8000000000000ll);
@@ -904,7 +929,7 @@ k_adj_observe(EphemDev E, AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
         double g[6] = {0, 0, 0, 0, 0, 0};
         for (int j = j0; j < j1; j++)
 #pragma unroll
-            for (int c = 0; c < 6; c++) g[c] += sh[w][j][1 + c];
+            for (int c = 0; c < 6; c++) g[c] += mine_sh[j][1 + c];
         double *dst = B.gjump + ((size_t)i * P.m + kb) * 6;
 #pragma unroll
         for (int c = 0; c < 6; c++) dst[c] = g[c];
@@ -1393,35 +1418,39 @@ cudaError_t launch_adjoint_last_epoch(const AdjProblem &P, int64_t i0, int64_t n
     return cudaGetLastError();
 }
 
+static int64_t forward_grid(int64_t nc, bool full)
+{
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (full) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adj_forward<true>, 128, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adj_forward<false>, 128, 0);
+    const int64_t persistent = (int64_t)(sms > 0 ? sms : 152) * (per_sm > 0 ? per_sm : 1);
+    const int64_t grid = blocks_for(nc, 128);
+    return grid < persistent ? grid : persistent;
+}
+
+int64_t adjoint_forward_lanes(int64_t nc, bool full) { return 128 * forward_grid(nc, full); }
+
 cudaError_t launch_adjoint_forward(const EphemDev &E, const ForceDev &F, const AdjBuffers &B,
                                    const AdjProblem &P, int64_t i0, int64_t nc,
                                    unsigned long long *next, cudaStream_t st,
                                    const int32_t *order)
 {
     if (nc <= 0) return cudaGetLastError();
-    int64_t grid = blocks_for(nc, 128);
-    int refill = 0;
-    if (next) {   // persistent grid with work stealing
-        cudaError_t e = cudaMemsetAsync(next, 0, sizeof(unsigned long long), st);
-        if (e != cudaSuccess) return e;
-        int dev = 0, sms = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (B.recx) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adj_forward<true>, 128, 0);
-        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adj_forward<false>, 128, 0);
-        const int64_t persistent = (int64_t)(sms > 0 ? sms : 152) * (per_sm > 0 ? per_sm : 1);
-        if (grid > persistent) grid = persistent;
-        refill = 1;
-    }
-    if (B.recx) k_adj_forward<true><<<(unsigned)grid, 128, 0, st>>>(E, F, B, P, i0, nc, next, refill, order);
-    else k_adj_forward<false><<<(unsigned)grid, 128, 0, st>>>(E, F, B, P, i0, nc, next, refill, order);
+    // persistent grid with work stealing
+    const cudaError_t e = cudaMemsetAsync(next, 0, sizeof(unsigned long long), st);
+    if (e != cudaSuccess) return e;
+    const int64_t grid = forward_grid(nc, B.recx != nullptr);
+    if (B.recx) k_adj_forward<true><<<(unsigned)grid, 128, 0, st>>>(E, F, B, P, i0, nc, next, order);
+    else k_adj_forward<false><<<(unsigned)grid, 128, 0, st>>>(E, F, B, P, i0, nc, next, order);
     return cudaGetLastError();
 }
 
 cudaError_t launch_adjoint_observe(const EphemDev &E, const AdjBuffers &B, const AdjProblem &P,
                                    int64_t i0, int64_t nc, cudaStream_t st)
 {
-    if (nc > 0) k_adj_observe<<<blocks_for(nc, 4), 128, 0, st>>>(E, B, P, i0, nc);
+    if (nc > 0) k_adj_observe<<<blocks_for(nc, 128 / P.m), 128, 0, st>>>(E, B, P, i0, nc);
     return cudaGetLastError();
 }
 

@@ -50,10 +50,14 @@ struct AdjBuffers {
                        // its records carry recx; 0: a body without terms, Newtonian
                        // records only
     int32_t *status;   // [nc]
+    double *planets;   // [7 n_bodies 6][lanes of the forward grid]: see attempt_sweep
 };
 
+// lanes of the forward pass's grid for chunks of nc bodies
+int64_t adjoint_forward_lanes(int64_t nc, bool full);
+
 cudaError_t upload_adjoint_tables(cudaStream_t st);
-// next != null: persistent grid with work stealing from the counter *next;
+// persistent grid with work stealing from the counter *next;
 // order != null: lanes take the chunk's bodies in that order
 cudaError_t launch_adjoint_forward(const EphemDev &E, const ForceDev &F, const AdjBuffers &B,
                                    const AdjProblem &P, int64_t i0, int64_t nc,

@@ -400,6 +400,15 @@ static __device__ __forceinline__ NgOut nongrav_terms(const EphemDev &E, const d
                                                       double x2, double v0, double v1, double v2,
                                                       double chi0);
 
+// The planets of one node of a step attempt as one lane sums them in the
+// attempt's first sweep (store) and reads them back in the others: element e
+// of body m at p[(6 m + e) stride].
+struct PlanetCache {
+    double *p;        // null: none
+    int64_t stride;
+    bool store;
+};
+
 // Full-FP64 acceleration.
 // detect (step start, off = 0): also record in enc the nearest planet within
 // kEncounterAu and its relative position; otherwise enc is read.
@@ -412,9 +421,11 @@ __device__ __forceinline__ int accel_fp64(const EphemDev &E, const ForceDev &F, 
                                           const double x[3], const double v[3], double a[3],
                                           Encounter &enc, const double dx[3], bool detect,
                                           double *J = nullptr, const kete_nongrav *ng = nullptr,
-                                          double *ng_chi = nullptr, double *helio = nullptr)
+                                          double *ng_chi = nullptr, double *helio = nullptr,
+                                          PlanetCache cache = PlanetCache{nullptr, 0, false})
 {
     Seg g = {0, 0.0};
+    const bool cached = cache.p && !cache.store;
     a[0] = a[1] = a[2] = 0.0;
     if (JAC) {
 #pragma unroll
@@ -425,14 +436,14 @@ __device__ __forceinline__ int accel_fp64(const EphemDev &E, const ForceDev &F, 
         enc.t0 = t0;
     }
     double best = kEncounterAu * kEncounterAu;
-    if (!row64 && !ephem_seg(E, t0, off, g)) return KETE_BODY_OUT_OF_SPAN;
+    if (!row64 && (!cached || ng) && !ephem_seg(E, t0, off, g)) return KETE_BODY_OUT_OF_SPAN;
     // per-thread ephemeris: one Chebyshev basis for all the bodies, in shared
     // memory (a column per thread)
     __shared__ double s_basis[2 * kBasisMax * kBasisLanes];
     ChebBasis basis;
     basis.T = s_basis + threadIdx.x;
     basis.dT = s_basis + kBasisMax * kBasisLanes + threadIdx.x;
-    const bool use_basis = !row64 && E.n_coef <= kBasisMax && threadIdx.x < kBasisLanes &&
+    const bool use_basis = !row64 && !cached && E.n_coef <= kBasisMax && threadIdx.x < kBasisLanes &&
                            blockDim.x <= kBasisLanes;
     if (use_basis) cheb_basis(E.n_coef, g.tau, (F.gr_mask & F.active_mask) != 0u, basis);
     for (int m = 0; m < E.n_bodies; m++) {
@@ -447,12 +458,24 @@ __device__ __forceinline__ int accel_fp64(const EphemDev &E, const ForceDev &F, 
 #pragma unroll
                 for (int q = 3; q < 6; q++) st[q] = __ldg(row64 + 6 * m + q);
             }
+        } else if (cached) {
+#pragma unroll
+            for (int q = 0; q < 3; q++) st[q] = cache.p[(6 * m + q) * cache.stride];
+            if (gr) {
+#pragma unroll
+                for (int q = 3; q < 6; q++) st[q] = cache.p[(6 * m + q) * cache.stride];
+            }
         } else if (use_basis) {
             const PlanetState o = cheb_state64b(E, m, g.s, basis, gr);
             st[0] = o.x; st[1] = o.y; st[2] = o.z;
             st[3] = o.vx; st[4] = o.vy; st[5] = o.vz;
         } else {
             cheb_state64(E, m, g.s, g.tau, st, gr);
+        }
+        if (cache.p && cache.store) {
+#pragma unroll
+            for (int q = 0; q < 6; q++)
+                if (q < 3 || gr) cache.p[(6 * m + q) * cache.stride] = st[q];
         }
         double r[3] = {x[0] - st[0], x[1] - st[1], x[2] - st[2]};
         if (detect) {

@@ -101,14 +101,16 @@ __device__ __forceinline__ int accel(const EphemDev &E, const ForceDev &F, doubl
                                      double as[3], Encounter &enc, const double dx[3], bool detect,
                                      double *jout = nullptr, const kete_nongrav *ng = nullptr,
                                      const float *vf = nullptr, double *ng_chi = nullptr,
-                                     double *helio = nullptr)
+                                     double *helio = nullptr,
+                                     PlanetCache cache = PlanetCache{nullptr, 0, false})
 {
     static_assert(!(JAC && MODE == KETE_MIXED), "Jacobian capture is FP64 only");
     if (MODE == KETE_MIXED)
         return accel_mixed(E, F, t0, off, row64, row32, close, x, v, a, as, enc, dx, detect, ng,
                            vf, ng_chi, helio);
     double J[6];
-    int st = accel_fp64<JAC>(E, F, t0, off, row64, x, v, a, enc, dx, detect, J, ng, ng_chi, helio);
+    int st = accel_fp64<JAC>(E, F, t0, off, row64, x, v, a, enc, dx, detect, J, ng, ng_chi, helio,
+                             cache);
     as[0] = a[0]; as[1] = a[1]; as[2] = a[2];
     if (JAC) {
 #pragma unroll
@@ -202,6 +204,8 @@ __device__ __forceinline__ void node_update(Attempt &A, const double Fn[3], cons
 // (max|db6|/max|a| < eps_pc), stopped improving (from the third sweep) or
 // reached max_iter sweeps.  JAC: every node evaluation also stores da/dx at
 // node n to jrec[6n..6n+5]; the last sweep's values remain.
+// planets (FP64, no rows): this lane's scratch of 7 E.n_bodies 6 doubles, pstride
+// apart, where the first sweep keeps the planets for the others.
 template <int MODE, bool JAC = false, bool V32 = false>
 __device__ __forceinline__ int attempt_sweep(const EphemDev &E, const ForceDev &F, double t,
                                              const double x0[3], const double v0[3],
@@ -209,7 +213,8 @@ __device__ __forceinline__ int attempt_sweep(const EphemDev &E, const ForceDev &
                                              uint32_t close, Encounter enc, Attempt &A, bool &done,
                                              Cnt &cnt, double *jrec = nullptr,
                                              const kete_nongrav *ng = nullptr,
-                                             double *ng_chi = nullptr)
+                                             double *ng_chi = nullptr, double *planets = nullptr,
+                                             int64_t pstride = 0)
 {
     const double h = A.h;
     double b6o[3] = {A.b[6][0], A.b[6][1], A.b[6][2]};
@@ -267,9 +272,11 @@ __device__ __forceinline__ int attempt_sweep(const EphemDev &E, const ForceDev &
         double Fn[3], Fs[3];
         const double *r64 = A.rows.r64 ? A.rows.r64 + n * A.rows.stride : nullptr;
         const float *r32 = A.rows.r32 ? A.rows.r32 + n * A.rows.stride : nullptr;
+        PlanetCache cache = {nullptr, pstride, A.it == 0};
+        if (planets) cache.p = planets + (int64_t)(n - 1) * E.n_bodies * 6 * pstride;
         int st = accel<MODE, JAC>(E, F, t, sh, r64, r32, close, xn, vn, Fn, Fs, enc, dxn,
                                      false, JAC ? jrec + 6 * n : nullptr, ng,
-                                     vel32 ? vnf : nullptr, ng_chi);
+                                     vel32 ? vnf : nullptr, ng_chi, nullptr, cache);
         cnt.evals++;
         if (r64) cnt.node_evals++;
         if (st != KETE_BODY_OK) return st;
@@ -605,28 +612,6 @@ __device__ __forceinline__ int step_end(const ForceDev &F, const Attempt &A, dou
     t = A.t_new;
     S.have_a0 = false;
     return KETE_BODY_OK;
-}
-
-// One whole step attempt of (x, v, t) toward `target` (t != target):
-// step_begin, corrector sweeps until done, step_end.
-// JAC: da/dx at the 8 nodes of the attempt go to jrec[6n..6n+5]; after an
-// accepted step they describe that step.
-template <int MODE, bool JAC = false>
-__device__ __forceinline__ int step_once(const EphemDev &E, const ForceDev &F, double x[3],
-                                         double v[3], double &t, double &dt, double target,
-                                         StepState &S, Cnt &cnt, double *jrec = nullptr)
-{
-    Attempt A;
-    int st = step_begin<MODE, JAC>(E, F, x, v, t, dt, target, S, A, cnt, jrec);
-    if (st != KETE_BODY_OK) return st;
-    for (;;) {
-        bool done = false;
-        st = attempt_sweep<MODE, JAC>(E, F, t, x, v, S.a0, S.as0, S.close, S.enc, A, done, cnt,
-                                         jrec, S.ng, &S.ng_chi);
-        if (st != KETE_BODY_OK) return st;
-        if (done) break;
-    }
-    return step_end<MODE, JAC>(F, A, x, v, t, dt, S, cnt);
 }
 
 // orient the carried step toward the next stop (|dt| kept; dt_init to start)
