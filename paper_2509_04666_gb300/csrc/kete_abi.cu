@@ -34,7 +34,7 @@ enum Slot {
     S_ORDER_SCAN, S_ORDER_N, S_ADJ_TEND, S_LEG_OUT,
     S_EXT_START, S_EXT_EX, S_EXT_TMP, S_EXT_FIRST, S_EXT_SUB, S_EXT_PARENT, S_EXT_CNT,
     S_EXT_OFF, S_EXT_CUR, S_EXT_GROUP, S_EXT_KEEP, S_EXT_KCNT, S_EXT_KOFF, S_ADJ_PHI, S_ADJ_RECX,
-    S_PRE_KEEP, S_PRE_N, S_ADJ_RICH, S_ADJ_PLANETS,
+    S_PRE_KEEP, S_PRE_N, S_ADJ_RICH, S_ADJ_PLANETS, S_ADJ_BFRAC,
     S_NSLOTS
 };
 
@@ -1466,6 +1466,13 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
         chunk = std::max<int64_t>(1, std::min<int64_t>(chunk, n));
         const int64_t n_chunks = (n + chunk - 1) / chunk;   // even chunks
         chunk = (n + n_chunks - 1) / n_chunks;
+        // few bodies: one warp per body (see takes_warps); more keep the lanes'
+        // step sequence (see step_factor)
+        WarpModel model;
+        const bool warps = !full && n <= kWarpBodies && F.max_iter >= 8 &&
+                           warp_model(ctx->E, F, model);
+        if (warps) F.eps_pc = kStartTighter * fm64.eps_pc;
+        const bool want_phi = jac || (warps && grad);
         AdjBuffers B;
         B.cap = cap;
         GET(S_ADJ_REC, (size_t)chunk * cap * kAdjRec, B.rec);
@@ -1476,7 +1483,9 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
         GET(S_ADJ_GJUMP, (size_t)chunk * m * 6, B.gjump);
         GET(S_ADJ_STATUS, chunk, B.status);
         B.phi = nullptr;
-        if (jac) GET(S_ADJ_PHI, (size_t)chunk * m * 36, B.phi);
+        B.bfrac = nullptr;
+        if (want_phi) GET(S_ADJ_PHI, (size_t)chunk * m * 36, B.phi);
+        if (want_phi || warps) GET(S_ADJ_BFRAC, (size_t)chunk * m, B.bfrac);
         B.recx = nullptr;
         B.rich = nullptr;
         if (full) {
@@ -1495,7 +1504,7 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
             const int64_t nc = std::min(chunk, n - i0);
             prop_event(ctx, true);
             int32_t *order = nullptr;
-            if (order_on) {   // most expensive bodies first (schedule only)
+            if (order_on && !warps) {   // most expensive bodies first (schedule only)
                 unsigned long long *order_n;
                 CUDA_TRY(launch_adjoint_last_epoch(P, i0, nc, t_end, ctx->stream));
                 // bodies with and without non-gravitational terms in separate
@@ -1505,16 +1514,18 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
                 if (r2 != KETE_OK) return r2;
                 launches += 1;
             }
-            CUDA_TRY(launch_adjoint_forward(ctx->E, F, B, P, i0, nc, next, ctx->stream, order));
+            if (warps) CUDA_TRY(launch_adjoint_forward_warp(ctx->E, F, model, B, P, i0, nc, ctx->stream));
+            else CUDA_TRY(launch_adjoint_forward(ctx->E, F, B, P, i0, nc, next, ctx->stream, order));
             prop_event(ctx, false);
-            if (jac) {
+            if (want_phi) {
                 CUDA_TRY(launch_adjoint_stm(B, P, i0, nc, ctx->stream));
                 launches++;
             }
             CUDA_TRY(launch_adjoint_observe(ctx->E, B, P, i0, nc, ctx->stream));
             launches += 2;
             if (grad) {
-                CUDA_TRY(launch_adjoint_backward(B, P, i0, nc, ctx->stream));
+                if (warps) CUDA_TRY(launch_adjoint_grad_phi(B, P, i0, nc, ctx->stream));
+                else CUDA_TRY(launch_adjoint_backward(B, P, i0, nc, ctx->stream));
                 launches++;
             }
         }

@@ -60,11 +60,13 @@ struct AdjTables {
     double sigf[9];
     double W1f[9][9];
     double W2f[9][9];
+    double Lf[9][9];   // l_k(s) = sum_p Lf[k][p] s^p on the forward samples
 };
 static __constant__ AdjTables g_adj;
 
 // Lagrange-basis integrals on 9 sample points sg (see AdjTables)
-static void fill_colloc(const long double sg[9], double sig[9], double W1[9][9], double W2[9][9])
+static void fill_colloc(const long double sg[9], double sig[9], double W1[9][9], double W2[9][9],
+                        double L[9][9] = nullptr)
 {
     for (int n = 0; n < 9; n++) sig[n] = (double)sg[n];
     for (int k = 0; k < 9; k++) {
@@ -79,6 +81,8 @@ static void fill_colloc(const long double sg[9], double sig[9], double W1[9][9],
             deg++;
             den *= (sg[k] - sg[j]);
         }
+        if (L)
+            for (int p = 0; p < 9; p++) L[k][p] = (double)(c[p] / den);
         for (int n = 0; n < 9; n++) {
             long double w1 = 0.0L, w2 = 0.0L, sp = sg[n];
             for (int p = 0; p <= 8; p++) {
@@ -103,7 +107,7 @@ static void fill_adj_tables(AdjTables &T)
     fill_colloc(sg, T.sig, T.W1, T.W2);
     for (int n = 0; n <= 7; n++) sg[n] = (long double)rt.h[n];
     sg[8] = 1.0L;
-    fill_colloc(sg, T.sigf, T.W1f, T.W2f);
+    fill_colloc(sg, T.sigf, T.W1f, T.W2f, T.Lf);
 }
 
 cudaError_t upload_adjoint_tables(cudaStream_t st)
@@ -117,32 +121,6 @@ cudaError_t upload_adjoint_tables(cudaStream_t st)
         filled = true;
     }
     return cudaMemcpyToSymbolAsync(g_adj, &T, sizeof(T), 0, cudaMemcpyHostToDevice, st);
-}
-
-// ---------------------------------------------------------------------------
-// batches of one body's observations (the <= span rule of Sec. 2)
-// ---------------------------------------------------------------------------
-// The batch starting at j0 ends before the returned index; tref = midpoint.
-__device__ __forceinline__ int next_batch(const kete_obs *o, int mi, int j0, double span,
-                                          double &tref)
-{
-    const double e0 = o[j0].epoch;
-    int j = j0;
-    while (j + 1 < mi) {
-        const double e = o[j + 1].epoch;
-        if (!(e == e0 || e - e0 < span)) break;
-        j++;
-    }
-    tref = 0.5 * (e0 + o[j].epoch);
-    return j + 1;
-}
-
-// observations in use: those before the first non-finite epoch
-__device__ __forceinline__ int obs_count(const kete_obs *o, int m)
-{
-    int mi = 0;
-    while (mi < m && isfinite(o[mi].epoch)) mi++;
-    return mi;
 }
 
 // ---------------------------------------------------------------------------
@@ -667,6 +645,7 @@ k_adj_forward(EphemDev E, ForceDev F, AdjBuffers B, AdjProblem P, int64_t i0, in
                                 y[3 + c] = v[c];
                             }
                             B.bidx[(size_t)i * P.m + W.kb] = count;
+                            if (B.bfrac) B.bfrac[(size_t)i * P.m + W.kb] = 0.0;
                             if (W.ckpt_ok && W.tc == W.tref) walk_next_ckpt(W, epoch0, P.ckpt);   // one stop
                             W.kb++;
                             if (W.kb < W.nb) W.j1 = next_batch(o, W.mi, W.j1, P.span, W.tref);
@@ -1062,7 +1041,40 @@ __device__ __forceinline__ const double *jac_sample_fwd(const double *r, const d
     return k == 8 ? r_next + 2 : r + 2 + 6 * k;
 }
 
-// One lane per body: the six columns (dx, dv) of Phi obey dx'' = J(t) dx.  Over
+// column c of Phi at (dx, dv), row-major 6x6 per batch
+__device__ __forceinline__ void store_column(double *ph, int c, const double dx[3], const double dv[3])
+{
+#pragma unroll
+    for (int r = 0; r < 3; r++) {
+        ph[r * 6 + c] = dx[r];
+        ph[(3 + r) * 6 + c] = dv[r];
+    }
+}
+
+// (dx, dv) at s in the step of size h from (dx0, dv0), F_k at the forward samples:
+// dx(s) = dx0 + s h dv0 + int int F, dv(s) = dv0 + (1/h) int F of the
+// interpolant through the samples, in powers of s.
+__device__ __forceinline__ void colloc_at(const double F[9][3], double h, double s,
+                                          const double dx0[3], const double dv0[3], double dx[3],
+                                          double dv[3])
+{
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        double p2 = 0.0, p1 = 0.0;
+#pragma unroll
+        for (int p = 8; p >= 0; p--) {
+            double cp = 0.0;
+#pragma unroll
+            for (int k = 0; k < 9; k++) cp = fma(g_adj.Lf[k][p], F[k][c], cp);
+            p2 = fma(p2, s, cp / ((p + 1.0) * (p + 2.0)));
+            p1 = fma(p1, s, cp / (p + 1.0));
+        }
+        dx[c] = fma(s * s, p2, fma(s * h, dv0[c], dx0[c]));
+        dv[c] = fma(s / h, p1, dv0[c]);
+    }
+}
+
+// One thread per body and column: the six columns (dx, dv) of Phi obey dx'' = J(t) dx.  Over
 // a recorded step of size h, with s = (t - t_start) / h and F_k = h^2 J_k dx_k
 // at the samples s_k (node 0..7, end):
 //   dx(s_n) = dx_0 + s_n h dv_0 + sum_k W2f[n][k] F_k,
@@ -1072,7 +1084,9 @@ __device__ __forceinline__ const double *jac_sample_fwd(const double *r, const d
 __global__ void __launch_bounds__(128)
 k_adj_stm(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = idx / 6;
+    const int c0 = (int)(idx % 6);
     if (i >= nc) return;
     const int st = B.status[i];
     if (st != KETE_BODY_OK) return;   // the observation kernel writes NaN rows
@@ -1081,20 +1095,16 @@ k_adj_stm(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
     const double *rec = B.rec + (size_t)i * B.cap * kAdjRec;
     const int32_t *bidx = B.bidx + (size_t)i * P.m;
     double *phi_out = B.phi + (size_t)i * P.m * 36;
-    for (int c0 = 0; c0 < 6; c0++) {
+    {
+        const double *bfrac = B.bfrac + (size_t)i * P.m;
         double dx[3] = {0, 0, 0}, dv[3] = {0, 0, 0};
         if (c0 < 3) dx[c0] = 1.0;
         else dv[c0 - 3] = 1.0;
         int kb = 0;
         for (int s = 0; s <= count - 1; s++) {
             // batches whose midpoint the chain reached after s steps
-            while (kb < nb && bidx[kb] == s) {
-                double *ph = phi_out + (size_t)kb * 36;
-#pragma unroll
-                for (int r = 0; r < 3; r++) {
-                    ph[r * 6 + c0] = dx[r];
-                    ph[(3 + r) * 6 + c0] = dv[r];
-                }
+            while (kb < nb && bidx[kb] == s && (bfrac[kb] == 0.0 || s == count - 1)) {
+                store_column(phi_out + (size_t)kb * 36, c0, dx, dv);
                 kb++;
             }
             if (s == count - 1) break;
@@ -1135,6 +1145,12 @@ k_adj_stm(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
                 }
                 if (delta <= 1e-16 * size) break;
             }
+// midpoints inside the step
+            for (; kb < nb && bidx[kb] == s; kb++) {
+                double xs[3], vs[3];
+                colloc_at(Fk, h, bfrac[kb], dx, dv, xs, vs);
+                store_column(phi_out + (size_t)kb * 36, c0, xs, vs);
+            }
 #pragma unroll
             for (int c = 0; c < 3; c++) {
                 double acc = 0.0;
@@ -1145,6 +1161,28 @@ k_adj_stm(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
             }
         }
     }
+}
+
+// dL/dy0 = sum over the batches of Phi^T dL/dy(t_ref): the gradient of few
+// bodies, whose state-transition matrices take six threads each where the
+// backward pass would run one lane.  Thread per body and component.
+__global__ void __launch_bounds__(128)
+k_adj_grad_phi(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
+{
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = idx / 6;
+    const int c = (int)(idx % 6);
+    if (i >= nc) return;
+    double g = 0.0;
+    if (B.status[i] != KETE_BODY_OK) g = __longlong_as_double(0x7ff8000000000000ll);
+    else
+        for (int k = B.nbat[i] - 1; k >= 0; k--) {
+            const double *phi = B.phi + ((size_t)i * P.m + k) * 36;
+            const double *j = B.gjump + ((size_t)i * P.m + k) * 6;
+#pragma unroll
+            for (int r = 0; r < 6; r++) g = fma(j[r], phi[6 * r + c], g);
+        }
+    P.grad[c * P.n + i0 + i] = g;
 }
 
 // ---------------------------------------------------------------------------
@@ -1308,7 +1346,9 @@ k_adj_backward_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 __global__ void __launch_bounds__(128)
 k_adj_stm_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = idx / 6;
+    const int c0 = (int)(idx % 6);
     if (i >= nc) return;
     if (B.status[i] != KETE_BODY_OK) return;   // the observation kernel writes NaN rows
     const int count = B.n_rec[i];
@@ -1317,19 +1357,15 @@ k_adj_stm_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
     const double *recx = B.rich[i] ? B.recx + (size_t)i * B.cap * kAdjRecX : nullptr;
     const int32_t *bidx = B.bidx + (size_t)i * P.m;
     double *phi_out = B.phi + (size_t)i * P.m * 36;
-    for (int c0 = 0; c0 < 6; c0++) {
+    {
+        const double *bfrac = B.bfrac + (size_t)i * P.m;
         double dx[3] = {0, 0, 0}, dv[3] = {0, 0, 0};
         if (c0 < 3) dx[c0] = 1.0;
         else dv[c0 - 3] = 1.0;
         int kb = 0;
         for (int s = 0; s <= count - 1; s++) {
-            while (kb < nb && bidx[kb] == s) {
-                double *ph = phi_out + (size_t)kb * 36;
-#pragma unroll
-                for (int q = 0; q < 3; q++) {
-                    ph[q * 6 + c0] = dx[q];
-                    ph[(3 + q) * 6 + c0] = dv[q];
-                }
+            while (kb < nb && bidx[kb] == s && (bfrac[kb] == 0.0 || s == count - 1)) {
+                store_column(phi_out + (size_t)kb * 36, c0, dx, dv);
                 kb++;
             }
             if (s == count - 1) break;
@@ -1383,6 +1419,12 @@ k_adj_stm_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
                                  F[n]);
                 }
                 if (delta <= 1e-16 * size) break;
+            }
+// midpoints inside the step
+            for (; kb < nb && bidx[kb] == s; kb++) {
+                double xs[3], vs[3];
+                colloc_at(F, h, bfrac[kb], dx, dv, xs, vs);
+                store_column(phi_out + (size_t)kb * 36, c0, xs, vs);
             }
 #pragma unroll
             for (int c = 0; c < 3; c++) {
@@ -1458,8 +1500,16 @@ cudaError_t launch_adjoint_stm(const AdjBuffers &B, const AdjProblem &P, int64_t
                                cudaStream_t st)
 {
     if (nc <= 0) return cudaGetLastError();
-    if (B.recx) k_adj_stm_full<<<blocks_for(nc, 128), 128, 0, st>>>(B, P, i0, nc);
-    else k_adj_stm<<<blocks_for(nc, 128), 128, 0, st>>>(B, P, i0, nc);
+    const int stm_block = nc < 4096 ? 32 : 128;   // few bodies: one warp to a block, spread over the SMs
+    if (B.recx) k_adj_stm_full<<<blocks_for(6 * nc, stm_block), stm_block, 0, st>>>(B, P, i0, nc);
+    else k_adj_stm<<<blocks_for(6 * nc, stm_block), stm_block, 0, st>>>(B, P, i0, nc);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_adjoint_grad_phi(const AdjBuffers &B, const AdjProblem &P, int64_t i0,
+                                    int64_t nc, cudaStream_t st)
+{
+    if (nc > 0) k_adj_grad_phi<<<blocks_for(6 * nc, 128), 128, 0, st>>>(B, P, i0, nc);
     return cudaGetLastError();
 }
 

@@ -41,7 +41,7 @@ struct AdjBuffers {
     double *yref;      // [nc][m][6] state at batch k's midpoint
     double *gjump;     // [nc][m][6] dL/dy(t_ref) of batch k
     double *phi;       // [nc][m][36] state-transition matrix at batch k's midpoint
-                       // (row-major, d y_r(t_ref) / d y0_c; only with P.jac)
+                       // (row-major, d y_r(t_ref) / d y0_c), or null
     double *recx;      // [nc][cap][8][18] per record and node: da/dx beyond the Newtonian
                        // part (9, row-major) and da/dv (9) -- the full force model's
                        // Jacobian (calls with non-gravitational terms); null: the
@@ -50,13 +50,46 @@ struct AdjBuffers {
                        // its records carry recx; 0: a body without terms, Newtonian
                        // records only
     int32_t *status;   // [nc]
+    double *bfrac;     // [nc][m] (with phi) where in step bidx[k] batch k's midpoint
+                       // lies, (t_ref - t_start) / h; 0: at the step's start
     double *planets;   // [7 n_bodies 6][lanes of the forward grid]: see attempt_sweep
 };
 
 // lanes of the forward pass's grid for chunks of nc bodies
 int64_t adjoint_forward_lanes(int64_t nc, bool full);
 
+// observations in use: those before the first non-finite epoch
+__device__ __forceinline__ int obs_count(const kete_obs *o, int m)
+{
+    int mi = 0;
+    while (mi < m && isfinite(o[mi].epoch)) mi++;
+    return mi;
+}
+
+// batches of one body's observations (the <= span rule of Sec. 2): the batch
+// starting at j0 ends before the returned index; tref = midpoint.
+__device__ __forceinline__ int next_batch(const kete_obs *o, int mi, int j0, double span,
+                                          double &tref)
+{
+    const double e0 = o[j0].epoch;
+    int j = j0;
+    while (j + 1 < mi) {
+        const double e = o[j + 1].epoch;
+        if (!(e == e0 || e - e0 < span)) break;
+        j++;
+    }
+    tref = 0.5 * (e0 + o[j].epoch);
+    return j + 1;
+}
+
 cudaError_t upload_adjoint_tables(cudaStream_t st);
+// kete_warp.cu: the forward pass with one warp per body, for few bodies without
+// non-gravitational terms: steps of
+// the size the step control proposes, the batch midpoints inside them from the
+// step polynomial (B.bfrac)
+cudaError_t launch_adjoint_forward_warp(const EphemDev &E, const ForceDev &F, const WarpModel &W,
+                                        const AdjBuffers &B, const AdjProblem &P, int64_t i0,
+                                        int64_t nc, cudaStream_t st);
 // persistent grid with work stealing from the counter *next;
 // order != null: lanes take the chunk's bodies in that order
 cudaError_t launch_adjoint_forward(const EphemDev &E, const ForceDev &F, const AdjBuffers &B,
@@ -69,6 +102,9 @@ cudaError_t launch_adjoint_last_epoch(const AdjProblem &P, int64_t i0, int64_t n
 cudaError_t launch_adjoint_observe(const EphemDev &E, const AdjBuffers &B, const AdjProblem &P,
                                    int64_t i0, int64_t nc, cudaStream_t st);
 cudaError_t launch_adjoint_backward(const AdjBuffers &B, const AdjProblem &P, int64_t i0,
+                                    int64_t nc, cudaStream_t st);
+// the gradient from the state-transition matrices (B.phi) and B.gjump
+cudaError_t launch_adjoint_grad_phi(const AdjBuffers &B, const AdjProblem &P, int64_t i0,
                                     int64_t nc, cudaStream_t st);
 // the state-transition matrix at every batch midpoint (B.phi), integrated
 // forward over the recorded steps

@@ -26,6 +26,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "kete_adjoint.h"
 #include "kete_step.cuh"
 
 namespace kete {
@@ -201,17 +202,53 @@ __device__ __forceinline__ float warp_max(float v)   // v >= 0 or NaN
     return __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(v)));
 }
 
-template <bool NG>
+// The Newtonian da/dx (newton_jacobian) at the lane's node from its masses,
+// summed over the group's four lanes.
+__device__ __forceinline__ void node_jacobian(const LaneMasses &M, const double x[3],
+                                              const double dx[3], int enc_slot,
+                                              const double d0[3], double J[6])
+{
+#pragma unroll
+    for (int q = 0; q < 6; q++) J[q] = 0.0;
+#pragma unroll
+    for (int s = 0; s < kSlots; s++) {
+        double d[3];
+#pragma unroll
+        for (int c = 0; c < 3; c++)
+            d[c] = enc_slot == s ? d0[c] + (dx[c] - M.p[s][c]) : x[c] - M.p[s][c];
+        newton_jacobian(M.mu[s], d, J);
+    }
+#pragma unroll
+    for (int q = 0; q < 6; q++) {
+        J[q] += __shfl_xor_sync(kFull, J[q], 1);
+        J[q] += __shfl_xor_sync(kFull, J[q], 2);
+    }
+}
+
+// the forward pass of an orbit fit (REC): its arrays and the chunk's first body
+struct WarpRecord {
+    AdjBuffers B;
+    AdjProblem P;
+    int64_t i0;
+};
+
+// REC: the bodies are those of an orbit fit.  The stops are each body's batch
+// midpoints, kept with the step each lies in, and every accepted step leaves
+// its epochs and the Newtonian da/dx at its nodes (see kete_adjoint.cu).
+template <bool NG, bool REC>
 __global__ void __launch_bounds__(32)
 k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
-                 const double *__restrict__ stops, const int32_t *__restrict__ stop_row,
-                 int n_stops, double *__restrict__ out, int64_t out_stride, int out_aos,
-                 int keep_on_fail, DevCounters *ctr, PropQueue q)
+                 const double *__restrict__ stops_in, const int32_t *__restrict__ stop_row,
+                 int n_stops_in, double *__restrict__ out, int64_t out_stride, int out_aos,
+                 int keep_on_fail, DevCounters *ctr, PropQueue q, WarpRecord R)
 {
+    __shared__ double mid[KETE_ADJ_MAX_OBS];
+    const double *stops = REC ? mid : stops_in;
+    int n_stops = n_stops_in;
     const int64_t n = cs.n;
     const int lane = threadIdx.x & 31, node = lane >> 2, r = lane & 3;
     const int rc = r < 3 ? r : 2;   // the coordinate this lane computes (lane 3: a copy of 2)
-    const unsigned long long n_items = q.list ? *q.list_n : (unsigned long long)n;
+    const unsigned long long n_items = !REC && q.list ? *q.list_n : (unsigned long long)n;
     Cnt cnt = {0, 0, 0, 0, 0};
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     const double inf = __longlong_as_double(0x7ff0000000000000ll);
@@ -245,12 +282,54 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
     // contracts what is left by ~1e-3, below the rounding of the positions
     const float tol = (float)(0.3 * F.eps_pc);
     for (unsigned long long item = blockIdx.x; item < n_items; item += gridDim.x) {
-        const int64_t i = q.list ? (int64_t)q.list[item] : (int64_t)item;
+        const int64_t i = !REC && q.list ? (int64_t)q.list[item] : (int64_t)item;
         // own coordinate of the step-start state
-        double x0 = cs.w[rc * n + i], v0 = cs.w[(3 + rc) * n + i];
-        double t = cs.w[6 * n + i], dt = cs.w[7 * n + i];
-        int status = cs.status[i];
-        int k = q.resume ? cs.kstop[i] : 0;
+        double x0, v0, t, dt = 0.0;
+        int status = KETE_BODY_OK, k = 0, count = 0;
+        double *rec = nullptr;
+        bool capped = false;
+        if (REC) {
+            const AdjProblem &P = R.P;
+            const int64_t gi = R.i0 + i;
+            const kete_obs *o = P.obs + gi * P.m;
+            x0 = P.states[rc * P.n + gi];
+            v0 = P.states[(3 + rc) * P.n + gi];
+            t = P.epochs[gi];
+            rec = R.B.rec + (size_t)i * R.B.cap * kAdjRec;
+            if (!__all_sync(kFull, isfinite(x0) && isfinite(v0) && isfinite(t)))
+                status = KETE_BODY_NONFINITE;
+            const int mi = obs_count(o, P.m);
+            bool sorted = true;
+            for (int j = 1; j < mi; j++) sorted = sorted && !(o[j].epoch < o[j - 1].epoch);
+            if (!sorted) {
+                if (lane == 0) atomicOr(&ctr->error_flags, 1 << 6);
+                status = KETE_BODY_NONFINITE;
+            }
+            n_stops = 0;
+            double last = t;
+            __syncwarp();
+            for (int j0 = 0; j0 < mi; n_stops++) {
+                j0 = next_batch(o, mi, j0, P.span, last);
+                if (lane == 0) mid[n_stops] = last;
+            }
+            __syncwarp();
+            // the checkpoint grid bounds no step here, but its stops count toward
+            // the limits as they do where the steps end at them
+            if (P.ckpt > 0.0 && last > t) {
+                const double ck = ceil((last - t) / P.ckpt) - 1.0;
+                if (ck >= (double)kAdjMaxCkpt) status = KETE_BODY_STEP_CAP;
+                else if (ck + n_stops > (double)(R.B.cap - 1)) capped = true;
+                count = 0;
+            }
+        } else {
+            x0 = cs.w[rc * n + i];
+            v0 = cs.w[(3 + rc) * n + i];
+            t = cs.w[6 * n + i];
+            dt = cs.w[7 * n + i];
+            status = cs.status[i];
+            k = q.resume ? cs.kstop[i] : 0;
+        }
+        const double epoch0 = t;
         const kete_nongrav *ng = (NG && F.nongrav) ? F.nongrav + i : nullptr;
         double ng_chi = 0.0;
         long long attempts = 0;
@@ -261,6 +340,21 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
         double d0[3] = {0.0, 0.0, 0.0};
         while (k < n_stops && status == KETE_BODY_OK) {
             const double next_stop = stops[k];
+            if (REC && t == next_stop) {
+                if (node == 0 && r < 3) {
+                    double *y = R.B.yref + ((size_t)i * R.P.m + k) * 6;
+                    y[r] = x0;
+                    y[3 + r] = v0;
+                }
+                if (lane == 0) {
+                    R.B.bidx[(size_t)i * R.P.m + k] = count;
+                    R.B.bfrac[(size_t)i * R.P.m + k] = 0.0;
+                }
+                k++;
+                attempts = 0;
+                have_a0 = false;
+                continue;
+            }
             if (t == next_stop) {
                 const int row = stop_row ? stop_row[k] : k;
                 if (node == 0 && r < 3 && row >= 0) {
@@ -501,6 +595,33 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
                 continue;
             }
             cnt.steps++;
+            if (REC) {   // the step's record: da/dx at the nodes of its final polynomial
+                double px = g[6] * wx[6];
+#pragma unroll
+                for (int m = 5; m >= 0; m--) px = fma(g[m], wx[m], px);
+                const double sh = s_n * h;
+                const double dxr = fma(sh * sh, fma(a0, 0.5, px), sh * v0);
+                double dx[3], xn[3], J[6];
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    dx[c] = __shfl_sync(kFull, dxr, (lane & ~3) + c);
+                    xn[c] = xs[c] + dx[c];
+                }
+                node_jacobian(M, xn, dx, enc_slot, d0, J);
+                if (count < R.B.cap - 1) {
+                    double *rr = rec + (size_t)count * kAdjRec;
+                    if (lane == 0) {
+                        rr[0] = t;
+                        rr[1] = t_new;
+                    }
+                    if (r < 3) {
+                        rr[2 + 6 * node + r] = r == 0 ? J[0] : r == 1 ? J[1] : J[2];
+                        rr[5 + 6 * node + r] = r == 0 ? J[3] : r == 1 ? J[4] : J[5];
+                    }
+                } else {
+                    capped = true;
+                }
+            }
             // stops inside the step, eight at a time (node group q takes stop k + q)
             if (fwd && !careful && stops[k] < t_new) {
                 double b[7];
@@ -513,7 +634,11 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
                 for (;;) {
                     const int kq = k + node;
                     const bool in = kq < n_stops && stops[kq] < t_new;
-                    const int row = in ? (stop_row ? stop_row[kq] : kq) : -1;
+                    const int row = in ? (!REC && stop_row ? stop_row[kq] : kq) : -1;
+                    if (REC && in && r == 3) {
+                        R.B.bidx[(size_t)i * R.P.m + kq] = count;
+                        R.B.bfrac[(size_t)i * R.P.m + kq] = (stops[kq] - t) / h;
+                    }
                     if (row >= 0 && r < 3) {
                         const double off = stops[kq] - t, s = off / h;
                         double px = 0.0, pv = 0.0;   // Horner in s
@@ -524,9 +649,10 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
                         }
                         px = fma(px, s, 0.5 * a0);
                         pv = fma(pv, s, a0);
-                        double *o = out_aos ? out + ((int64_t)row * out_stride + i) * 6
-                                            : out + (int64_t)row * 6 * out_stride + i;
-                        const int64_t sd = out_aos ? 1 : out_stride;
+                        double *o = REC ? R.B.yref + ((size_t)i * R.P.m + row) * 6
+                                    : out_aos ? out + ((int64_t)row * out_stride + i) * 6
+                                              : out + (int64_t)row * 6 * out_stride + i;
+                        const int64_t sd = REC || out_aos ? 1 : out_stride;
                         o[r * sd] = x0 + fma(off * off, px, off * v0);
                         o[(3 + r) * sd] = fma(off, pv, v0);
                     }
@@ -540,6 +666,36 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
             v0 = v1;
             t = t_new;
             have_a0 = false;
+            if (REC && count < R.B.cap - 1) count++;
+        }
+        if (REC) {
+            if (R.P.ckpt > 0.0 && t > epoch0 &&
+                count + n_stops + ceil((t - epoch0) / R.P.ckpt) - 1.0 > (double)(R.B.cap - 1))
+                capped = true;
+            if (status == KETE_BODY_OK && !capped) {   // da/dx at the final state closes the last step
+                const bool inside = lane_planets(E, W, t, 0.0, M);
+                const double zero[3] = {0.0, 0.0, 0.0};
+                const double xs[3] = {__shfl_sync(kFull, x0, 0), __shfl_sync(kFull, x0, 1),
+                                      __shfl_sync(kFull, x0, 2)};
+                double J[6];
+                node_jacobian(M, xs, zero, -1, zero, J);
+                if (!__all_sync(kFull, inside)) status = KETE_BODY_OUT_OF_SPAN;
+                if (lane == 0) {
+                    double *rr = rec + (size_t)count * kAdjRec;
+                    rr[0] = t;
+                    rr[1] = t;
+#pragma unroll
+                    for (int c = 0; c < 6; c++) rr[2 + c] = J[c];
+                }
+                count++;
+            }
+            if (status == KETE_BODY_OK && capped) status = KETE_BODY_ADJ_CAP;
+            if (lane == 0) {
+                R.B.n_rec[i] = status == KETE_BODY_OK ? count : 0;
+                R.B.nbat[i] = n_stops;
+                R.B.status[i] = status;
+            }
+            continue;
         }
         // a failed body: no state at the remaining stops
         if (status != KETE_BODY_OK && !keep_on_fail)
@@ -570,22 +726,39 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
     }
 }
 
+static unsigned warp_grid(int64_t n)
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t most = (int64_t)(sms > 0 ? sms : 152) * 8;
+    return (unsigned)(n < most ? n : most);
+}
+
+cudaError_t launch_adjoint_forward_warp(const EphemDev &E, const ForceDev &F, const WarpModel &W,
+                                        const AdjBuffers &B, const AdjProblem &P, int64_t i0,
+                                        int64_t nc, cudaStream_t st)
+{
+    if (nc <= 0) return cudaGetLastError();
+    ChainState cs{};
+    cs.n = nc;
+    k_propagate_warp<false, true><<<warp_grid(nc), 32, 0, st>>>(
+        E, F, W, cs, nullptr, nullptr, 0, nullptr, 0, 0, 0, P.ctr, PropQueue{}, WarpRecord{B, P, i0});
+    return cudaGetLastError();
+}
+
 cudaError_t launch_propagate_warp(const EphemDev &E, const ForceDev &F, const WarpModel &W,
                                   ChainState cs, const double *stops, const int32_t *row,
                                   int n_stops, double *out, int64_t stride, bool keep_on_fail,
                                   DevCounters *ctr, cudaStream_t st, PropQueue q, bool out_aos)
 {
     if (cs.n <= 0 || n_stops <= 0) return cudaGetLastError();
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t most = (int64_t)(sms > 0 ? sms : 152) * 8;
-    const unsigned grid = (unsigned)(cs.n < most ? cs.n : most);
+    const unsigned grid = warp_grid(cs.n);
     const int aos = out_aos ? 1 : 0, kof = keep_on_fail ? 1 : 0;
     if (F.nongrav)
-        k_propagate_warp<true><<<grid, 32, 0, st>>>(E, F, W, cs, stops, row, n_stops, out, stride, aos, kof, ctr, q);
+        k_propagate_warp<true, false><<<grid, 32, 0, st>>>(E, F, W, cs, stops, row, n_stops, out, stride, aos, kof, ctr, q, WarpRecord{});
     else
-        k_propagate_warp<false><<<grid, 32, 0, st>>>(E, F, W, cs, stops, row, n_stops, out, stride, aos, kof, ctr, q);
+        k_propagate_warp<false, false><<<grid, 32, 0, st>>>(E, F, W, cs, stops, row, n_stops, out, stride, aos, kof, ctr, q, WarpRecord{});
     return cudaGetLastError();
 }
 
