@@ -934,6 +934,18 @@ __device__ __forceinline__ void jmul(const double *J, const double m[3], double 
     out[2] = fma(j2, m[0], fma(j4, m[1], j5 * m[2]));
 }
 
+// The sweeps of a collocation system have converged when the step end's change
+// falls below its rounding, or will at the next sweep: the changes shrink by
+// a fixed factor, so the next one is about delta^2 / before.  (The first test
+// alone is often never met -- the last bits keep flipping -- and cost up to 12
+// sweeps where 4 had converged.)
+__device__ __forceinline__ bool colloc_done(double delta, double size, double &before)
+{
+    const bool done = delta <= 1e-16 * size || delta * delta <= 1e-16 * size * before;
+    before = delta;
+    return done;
+}
+
 __global__ void __launch_bounds__(128)
 k_adj_backward(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 {
@@ -972,17 +984,22 @@ k_adj_backward(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
         const double h2 = h * h;
         // s-derivative at the step end: d mu / ds = -h d mu / dt
         const double q0[3] = {-h * mud[0], -h * mud[1], -h * mud[2]};
-        double Fk[9][3], mk[9][3];
+        double Fk[9][3], m8[3];
 #pragma unroll
         for (int k = 0; k < 9; k++) {
+            double mk[3];
 #pragma unroll
-            for (int c = 0; c < 3; c++) mk[k][c] = fma(g_adj.sig[k], q0[c], mu[c]);
-            jmul(jac_sample(r, rn, k), mk[k], Fk[k]);
+            for (int c = 0; c < 3; c++) mk[c] = fma(g_adj.sig[k], q0[c], mu[c]);
+            jmul(jac_sample(r, rn, k), mk, Fk[k]);
 #pragma unroll
-            for (int c = 0; c < 3; c++) Fk[k][c] *= h2;
+            for (int c = 0; c < 3; c++) {
+                Fk[k][c] *= h2;
+                m8[c] = mk[c];
+            }
         }
-        // Picard iteration of the collocation equations (a linear system with
-        // contraction ~ h^2 |J|); at most 12 sweeps
+        // Gauss-Seidel sweeps of the collocation equations (a linear system with
+        // contraction ~ h^2 |J|); at most 12
+        double before = 0.0;
         for (int it = 0; it < 12; it++) {
             double delta = 0.0, size = 0.0;
 #pragma unroll
@@ -998,20 +1015,16 @@ k_adj_backward(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
                 if (k == 8) {
 #pragma unroll
                     for (int c = 0; c < 3; c++) {
-                        delta = fmax(delta, fabs(nm[c] - mk[8][c]));
+                        delta = fmax(delta, fabs(nm[c] - m8[c]));
                         size = fmax(size, fabs(nm[c]));
+                        m8[c] = nm[c];
                     }
                 }
-#pragma unroll
-                for (int c = 0; c < 3; c++) mk[k][c] = nm[c];
-            }
-#pragma unroll
-            for (int k = 1; k < 9; k++) {
-                jmul(jac_sample(r, rn, k), mk[k], Fk[k]);
+                jmul(jac_sample(r, rn, k), nm, Fk[k]);
 #pragma unroll
                 for (int c = 0; c < 3; c++) Fk[k][c] *= h2;
             }
-            if (delta <= 1e-16 * size) break;
+            if (colloc_done(delta, size, before)) break;
         }
         double q8[3];
 #pragma unroll
@@ -1020,7 +1033,7 @@ k_adj_backward(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 #pragma unroll
             for (int j = 0; j < 9; j++) acc = fma(g_adj.W1[8][j], Fk[j][c], acc);
             q8[c] = acc;
-            mu[c] = mk[8][c];
+            mu[c] = m8[c];
             mud[c] = -q8[c] / h;
         }
     }
@@ -1066,8 +1079,8 @@ __device__ __forceinline__ void colloc_at(const double F[9][3], double h, double
             double cp = 0.0;
 #pragma unroll
             for (int k = 0; k < 9; k++) cp = fma(g_adj.Lf[k][p], F[k][c], cp);
-            p2 = fma(p2, s, cp / ((p + 1.0) * (p + 2.0)));
-            p1 = fma(p1, s, cp / (p + 1.0));
+            p2 = fma(p2, s, cp * (1.0 / ((p + 1.0) * (p + 2.0))));
+            p1 = fma(p1, s, cp * (1.0 / (p + 1.0)));
         }
         dx[c] = fma(s * s, p2, fma(s * h, dv0[c], dx0[c]));
         dv[c] = fma(s / h, p1, dv0[c]);
@@ -1079,7 +1092,7 @@ __device__ __forceinline__ void colloc_at(const double F[9][3], double h, double
 // at the samples s_k (node 0..7, end):
 //   dx(s_n) = dx_0 + s_n h dv_0 + sum_k W2f[n][k] F_k,
 //   dv(1)   = dv_0 + (1/h) sum_k W1f[8][k] F_k,
-// solved by Picard iteration (contraction ~ h^2 |J|, at most 12 sweeps).
+// solved by Gauss-Seidel sweeps (contraction ~ h^2 |J|, at most 12).
 // Phi is stored at each batch midpoint when the chain reaches it.
 __global__ void __launch_bounds__(128)
 k_adj_stm(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
@@ -1112,40 +1125,44 @@ k_adj_stm(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
             const double *rn = r + kAdjRec;
             const double h = __ldg(r + 1) - __ldg(r);
             const double h2 = h * h;
-            double xk[9][3], Fk[9][3];
+            double Fk[9][3], x8[3];
 #pragma unroll
             for (int k = 0; k < 9; k++) {
+                double xk[3];
 #pragma unroll
-                for (int c = 0; c < 3; c++) xk[k][c] = fma(g_adj.sigf[k] * h, dv[c], dx[c]);
-                jmul(jac_sample_fwd(r, rn, k), xk[k], Fk[k]);
+                for (int c = 0; c < 3; c++) xk[c] = fma(g_adj.sigf[k] * h, dv[c], dx[c]);
+                jmul(jac_sample_fwd(r, rn, k), xk, Fk[k]);
 #pragma unroll
-                for (int c = 0; c < 3; c++) Fk[k][c] *= h2;
+                for (int c = 0; c < 3; c++) {
+                    Fk[k][c] *= h2;
+                    x8[c] = xk[c];
+                }
             }
+            double before = 0.0;
             for (int it = 0; it < 12; it++) {
                 double delta = 0.0, size = 0.0;
 #pragma unroll
                 for (int k = 1; k < 9; k++) {
+                    double xk[3];
 #pragma unroll
                     for (int c = 0; c < 3; c++) {
                         double acc = fma(g_adj.sigf[k] * h, dv[c], dx[c]);
 #pragma unroll
                         for (int j = 0; j < 9; j++) acc = fma(g_adj.W2f[k][j], Fk[j][c], acc);
                         if (k == 8) {
-                            delta = fmax(delta, fabs(acc - xk[8][c]));
+                            delta = fmax(delta, fabs(acc - x8[c]));
                             size = fmax(size, fabs(acc));
+                            x8[c] = acc;
                         }
-                        xk[k][c] = acc;
+                        xk[c] = acc;
                     }
-                }
-#pragma unroll
-                for (int k = 1; k < 9; k++) {
-                    jmul(jac_sample_fwd(r, rn, k), xk[k], Fk[k]);
+                    jmul(jac_sample_fwd(r, rn, k), xk, Fk[k]);
 #pragma unroll
                     for (int c = 0; c < 3; c++) Fk[k][c] *= h2;
                 }
-                if (delta <= 1e-16 * size) break;
+                if (colloc_done(delta, size, before)) break;
             }
-// midpoints inside the step
+            // midpoints inside the step
             for (; kb < nb && bidx[kb] == s; kb++) {
                 double xs[3], vs[3];
                 colloc_at(Fk, h, bfrac[kb], dx, dv, xs, vs);
@@ -1157,7 +1174,7 @@ k_adj_stm(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 #pragma unroll
                 for (int j = 0; j < 9; j++) acc = fma(g_adj.W1f[8][j], Fk[j][c], acc);
                 dv[c] += acc / h;
-                dx[c] = xk[8][c];
+                dx[c] = x8[c];
             }
         }
     }
@@ -1296,6 +1313,7 @@ k_adj_backward_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 #pragma unroll
                 for (int c = 0; c < 3; c++) m8[c] = m[c];
         }
+        double before = 0.0;
         for (int it = 0; it < 16; it++) {
             double delta = 0.0, size = 0.0;
 #pragma unroll
@@ -1319,7 +1337,7 @@ k_adj_backward_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
                 }
                 adj_rhs_full(jac_sample(r, rn, n), jacx_sample(rx, rxn, n), h, m, G[n], H[n]);
             }
-            if (delta <= 1e-16 * size) break;
+            if (colloc_done(delta, size, before)) break;
         }
 #pragma unroll
         for (int c = 0; c < 3; c++) {
@@ -1390,6 +1408,7 @@ k_adj_stm_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
                         v8[c] = dv[c];
                     }
             }
+            double before = 0.0;
             for (int it = 0; it < 16; it++) {
                 double delta = 0.0, size = 0.0;
 #pragma unroll
@@ -1418,7 +1437,7 @@ k_adj_stm_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
                     var_rhs_full(jac_sample_fwd(r, rn, n), jacx_sample_fwd(rx, rxn, n), h, xn, vn,
                                  F[n]);
                 }
-                if (delta <= 1e-16 * size) break;
+                if (colloc_done(delta, size, before)) break;
             }
 // midpoints inside the step
             for (; kb < nb && bidx[kb] == s; kb++) {

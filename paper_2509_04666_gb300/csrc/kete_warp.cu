@@ -644,8 +644,8 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
                         double px = 0.0, pv = 0.0;   // Horner in s
 #pragma unroll
                         for (int m = 6; m >= 0; m--) {
-                            px = fma(px, s, b[m] / ((m + 2.0) * (m + 3.0)));
-                            pv = fma(pv, s, b[m] / (m + 2.0));
+                            px = fma(px, s, b[m] * (1.0 / ((m + 2.0) * (m + 3.0))));
+                            pv = fma(pv, s, b[m] * (1.0 / (m + 2.0)));
                         }
                         px = fma(px, s, 0.5 * a0);
                         pv = fma(pv, s, a0);
