@@ -537,6 +537,7 @@ static int propagate_launch(kete_ctx *ctx, const ForceDev &F, ChainState cs, dou
 static const int kGridLen[kGridLens] = {1,  2,  3,  4,  5,  6,  7,  8,  9,  10, 11, 12, 13,
                                         14, 15, 16, 18, 20, 22, 24, 28, 32, 40, 48, 64};
 constexpr int kGridUnits = 512;   // units of one grid: 512 x 25 steps x 9 bodies are 66 MB of rows
+constexpr double kGridMaxLaunches = 4096.0;   // grids of one call (5,700 years); longer spans take plain steps
 // The grid of one launch: points pts[0..J] (host, monotonic).  single: steps
 // of one unit only.
 static int make_grid(kete_ctx *ctx, const std::vector<double> &pts, double unit, bool single,
@@ -598,9 +599,16 @@ static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const doub
     if (few) use_grid = false;
     const double unit = leg_days > 0.0 ? leg_days : 1.0;
     double start = t_from;
-    const bool forward = n_stops > 1 ? stops[n_stops - 1] > stops[0] : stops[0] > t_from;
-    if (use_grid && (!std::isfinite(t_from) || (n_stops > 1 && t_from > stops[0]))) start = stops[0];
-    if (use_grid && !(stops[n_stops - 1] != start)) use_grid = false;
+    const double last = stops[n_stops - 1];
+    if (!std::isfinite(t_from) || (last > stops[0] && t_from > stops[0])) start = stops[0];
+    const bool forward = last > start;
+    if (last == start) use_grid = false;
+    if (leg_days == 0.0) {
+        // a target off the table fails every body; spans of millennia (and chains
+        // with stops far off the table) would be cut into too many launches
+        if (n_stops == 1 && !(last >= ctx->E.t_start && last <= ctx->E.t_end)) use_grid = false;
+        if (!(std::fabs(last - start) <= kGridMaxLaunches * kGridUnits * unit)) use_grid = false;
+    }
     if (use_grid) {
         // internal marks where a gap exceeds one launch
         std::vector<double> m2;

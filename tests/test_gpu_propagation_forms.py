@@ -148,3 +148,27 @@ def test_stops_before_a_failure_are_kept(K, pop, form):
     status = K.propagate(st, ep, end + 3.0)
     assert (status.cpu().numpy() == kete.BODY_OUT_OF_SPAN).all()
     assert np.array_equal(st.cpu().numpy(), states) and (ep.cpu().numpy() == epochs).all()
+
+
+@pytest.mark.parametrize("target", [1e15, -1e15])
+def test_target_far_off_the_table(K, pop, target):
+    """More bodies than the warp form takes, a target no grid of steps could
+    reach: every body is out of span, as with few bodies, and stops on the
+    table before such a stop still hold."""
+    from paper_2509_04666_gb300 import kete
+    w, states = pop
+    many = np.tile(states[:, :20], (1, 500))
+    epochs = np.full(many.shape[1], W.T0)
+    K.load_ephem(w.ephem.to_bytes())
+    st, ep = _dev(many), _dev(epochs)
+    status = K.propagate(st, ep, target)
+    assert (status.cpu().numpy() == kete.BODY_OUT_OF_SPAN).all()
+    assert np.array_equal(st.cpu().numpy(), many) and (ep.cpu().numpy() == epochs).all()
+    if target > 0:
+        out, status = K.propagate_stops(_dev(many), _dev(epochs), np.array([W.T0 + 1.0, target]))
+        out = out.cpu().numpy()
+        assert (status.cpu().numpy() == kete.BODY_OUT_OF_SPAN).all() and np.isnan(out[1]).all()
+        orc = O.Oracle(w.ephem.to_bytes())
+        for i in range(20):
+            rc, ref, _ = orc.propagate_stops(orc.force_model(), states[:, i], W.T0, [W.T0 + 1.0])
+            assert rc == 0 and np.abs(out[0, :3, i] - ref[0, :3]).max() < TOL
