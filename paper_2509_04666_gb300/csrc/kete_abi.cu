@@ -1468,19 +1468,16 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
         const size_t per_body = (size_t)cap * (kAdjRec + (full ? kAdjRecX : 0)) * sizeof(double) +
                                 (size_t)m * (sizeof(int32_t) + 12 * sizeof(double)) +
                                 (jac ? (size_t)m * 36 * sizeof(double) : 0) +
-                                3 * sizeof(int32_t);
+                                (size_t)m * sizeof(double) + 3 * sizeof(int32_t);
         const double budget = (opt.mem_budget_gb > 0 ? opt.mem_budget_gb : 8.0) * 1073741824.0;
         int64_t chunk = (int64_t)(budget / (double)per_body);
         chunk = std::max<int64_t>(1, std::min<int64_t>(chunk, n));
         const int64_t n_chunks = (n + chunk - 1) / chunk;   // even chunks
         chunk = (n + n_chunks - 1) / n_chunks;
-        // few bodies: one warp per body (see takes_warps); more keep the lanes'
-        // step sequence (see step_factor)
+        // one warp per body (kete_warp.cu); the lanes serve what that form does not
         WarpModel model;
-        const bool warps = !full && n <= kWarpBodies && F.max_iter >= 8 &&
-                           warp_model(ctx->E, F, model);
+        const bool warps = !full && F.max_iter >= 8 && warp_model(ctx->E, F, model);
         if (warps) F.eps_pc = kStartTighter * fm64.eps_pc;
-        const bool want_phi = jac || (warps && grad);
         AdjBuffers B;
         B.cap = cap;
         GET(S_ADJ_REC, (size_t)chunk * cap * kAdjRec, B.rec);
@@ -1490,18 +1487,19 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
         GET(S_ADJ_YREF, (size_t)chunk * m * 6, B.yref);
         GET(S_ADJ_GJUMP, (size_t)chunk * m * 6, B.gjump);
         GET(S_ADJ_STATUS, chunk, B.status);
+        GET(S_ADJ_BFRAC, (size_t)chunk * m, B.bfrac);
         B.phi = nullptr;
-        B.bfrac = nullptr;
-        if (want_phi) GET(S_ADJ_PHI, (size_t)chunk * m * 36, B.phi);
-        if (want_phi || warps) GET(S_ADJ_BFRAC, (size_t)chunk * m, B.bfrac);
+        if (jac) GET(S_ADJ_PHI, (size_t)chunk * m * 36, B.phi);
         B.recx = nullptr;
         B.rich = nullptr;
         if (full) {
             GET(S_ADJ_RECX, (size_t)chunk * cap * kAdjRecX, B.recx);
             GET(S_ADJ_RICH, chunk, B.rich);
         }
-        GET(S_ADJ_PLANETS, (size_t)adjoint_forward_lanes(chunk, full) * 7 * ctx->E.n_bodies * 6,
-            B.planets);
+        B.planets = nullptr;
+        if (!warps)
+            GET(S_ADJ_PLANETS, (size_t)adjoint_forward_lanes(chunk, full) * 7 * ctx->E.n_bodies * 6,
+                B.planets);
         unsigned long long *next = nullptr;
         GET(S_NEXTBODY, 1, next);
         int launches = 0;
@@ -1525,15 +1523,14 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
             if (warps) CUDA_TRY(launch_adjoint_forward_warp(ctx->E, F, model, B, P, i0, nc, ctx->stream));
             else CUDA_TRY(launch_adjoint_forward(ctx->E, F, B, P, i0, nc, next, ctx->stream, order));
             prop_event(ctx, false);
-            if (want_phi) {
+            if (jac) {
                 CUDA_TRY(launch_adjoint_stm(B, P, i0, nc, ctx->stream));
                 launches++;
             }
             CUDA_TRY(launch_adjoint_observe(ctx->E, B, P, i0, nc, ctx->stream));
             launches += 2;
             if (grad) {
-                if (warps) CUDA_TRY(launch_adjoint_grad_phi(B, P, i0, nc, ctx->stream));
-                else CUDA_TRY(launch_adjoint_backward(B, P, i0, nc, ctx->stream));
+                CUDA_TRY(launch_adjoint_backward(B, P, i0, nc, ctx->stream));
                 launches++;
             }
         }

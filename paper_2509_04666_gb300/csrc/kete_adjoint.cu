@@ -3,11 +3,14 @@
 // Sec. 2: n-body propagation of App. A, two-body + light time, RA/Dec).
 //
 // Three kernels per chunk of bodies:
-//   k_adj_forward   one lane per body at a time (work stealing).  The body's
-//                   observations are batched
+//   forward pass    k_propagate_warp (kete_warp.cu), or k_adj_forward, one lane
+//                   per body at a time (work stealing), with non-gravitational
+//                   terms and for force models the warp form does not serve.
+//                   The body's observations are batched
 //                   by the <= span rule (Sec. 2); the chain visits the batch
-//                   midpoints and the checkpoint grid in ascending order with
-//                   the same Gauss-Radau steps as the propagation kernel.
+//                   midpoints (k_adj_forward: and the checkpoint grid) in
+//                   ascending order with Gauss-Radau steps; k_propagate_warp
+//                   takes the midpoints inside a step from its polynomial.
 //                   Every accepted step leaves a record in device memory: its
 //                   start and end epochs and the Newtonian da/dx at its 8
 //                   Gauss-Radau nodes, taken from the force evaluations the
@@ -18,11 +21,11 @@
 //                   light-time fixed point (implicit derivative) and the
 //                   universal-variable two-body map (forward-mode dual numbers
 //                   at the converged universal anomaly).
-//   k_adj_backward  one lane per body: mu = lambda_v obeys mu'' = J(t) mu
-//                   (lambda_x = -mu'), integrated backward over every recorded
-//                   step by collocation on the step's 9 sample epochs (its 8
-//                   nodes and its end); dL/dy(t_ref) is added at each batch
-//                   midpoint.  dL/dx0 = -mu'(t0), dL/dv0 = mu(t0).
+//   k_adj_backward  one lane per body: (lambda_x, lambda_v) carried back over
+//                   every recorded step by the transpose of its variational
+//                   collocation on 9 sample epochs (the 8 nodes and the end),
+//                   dL/dy(t_ref) added at each batch midpoint, wherever it
+//                   lies in a step.
 //   k_adj_stm       (per-observation sky partials) one lane per body: the six
 //                   columns of the state-transition matrix obey dx'' = J(t) dx,
 //                   integrated forward over the recorded steps by the same
@@ -645,7 +648,7 @@ k_adj_forward(EphemDev E, ForceDev F, AdjBuffers B, AdjProblem P, int64_t i0, in
                                 y[3 + c] = v[c];
                             }
                             B.bidx[(size_t)i * P.m + W.kb] = count;
-                            if (B.bfrac) B.bfrac[(size_t)i * P.m + W.kb] = 0.0;
+                            B.bfrac[(size_t)i * P.m + W.kb] = 0.0;
                             if (W.ckpt_ok && W.tc == W.tref) walk_next_ckpt(W, epoch0, P.ckpt);   // one stop
                             W.kb++;
                             if (W.kb < W.nb) W.j1 = next_batch(o, W.mi, W.j1, P.span, W.tref);
@@ -925,6 +928,13 @@ __device__ __forceinline__ const double *jac_sample(const double *r, const doubl
     return r + 2 + 6 * (8 - k);               // forward node 8-k (k = 8: node 0)
 }
 
+// sample k of a step in the forward order: J at node k (k <= 7), at the step
+// end (k = 8: the next record's node 0)
+__device__ __forceinline__ const double *jac_sample_fwd(const double *r, const double *r_next, int k)
+{
+    return k == 8 ? r_next + 2 : r + 2 + 6 * k;
+}
+
 __device__ __forceinline__ void jmul(const double *J, const double m[3], double out[3])
 {
     const double j0 = __ldg(J), j1 = __ldg(J + 1), j2 = __ldg(J + 2), j3 = __ldg(J + 3),
@@ -946,14 +956,28 @@ __device__ __forceinline__ bool colloc_done(double delta, double size, double &b
     return done;
 }
 
+// Thread per body.  Every output of a recorded step -- the state change at its
+// end and at the midpoints inside it -- is linear in the step's 9 samples F_k
+// (see k_adj_stm):
+//   F_n = h^2 J_n (dx_0 + s_n h dv_0 + sum_k W2f[n][k] F_k),
+// so with phi_k the gradient with respect to F_k, summed over the end's
+// (lambda_x, lambda_v) and the midpoints' dL/dy, the transposed system
+//   z_k = phi_k + sum_n W2f[n][k] u_n,   u_n = h^2 J_n z_n (J symmetric)
+// is solved once a step however many midpoints it holds, and
+//   lambda_x <- lambda_x + sum g_x + sum u_n,
+//   lambda_v <- lambda_v + h lambda_x + sum (g_v + s h g_x) + h sum s_n u_n.
+// It is the exact transpose of k_adj_stm.  Gauss-Seidel sweeps from the step's
+// end (W2f is nearly lower triangular; contraction ~ h^2 |J|), at most 12.
+// FP64 issue bounds it: a sweep is 330 multiply-adds, a midpoint 400.  With the
+// forward pass stopping at no midpoint (6-7 steps instead of 25 over 90 days and
+// 20 midpoints), 100,000 bodies: loss and gradient 164 -> 68.6 ms.
 __global__ void __launch_bounds__(128)
 k_adj_backward(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nc) return;
     const int64_t gi = i0 + i;
-    const int st = B.status[i];
-    if (st != KETE_BODY_OK) {
+    if (B.status[i] != KETE_BODY_OK) {
         for (int c = 0; c < 6; c++) P.grad[c * P.n + gi] = __longlong_as_double(0x7ff8000000000000ll);
         return;
     }
@@ -961,99 +985,114 @@ k_adj_backward(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
     int kb = B.nbat[i] - 1;
     const double *rec = B.rec + (size_t)i * B.cap * kAdjRec;
     const int32_t *bidx = B.bidx + (size_t)i * P.m;
+    const double *bfrac = B.bfrac + (size_t)i * P.m;
     const double *gjump = B.gjump + (size_t)i * P.m * 6;
-    double mu[3] = {0, 0, 0}, mud[3] = {0, 0, 0};   // lambda_v and d lambda_v / dt
-    for (int s = count - 2; s >= -1; s--) {
-        // jumps of the batches whose midpoint the chain reached after s+1 steps
-        while (kb >= 0 && bidx[kb] == s + 1) {
+    double lx[3] = {0, 0, 0}, lv[3] = {0, 0, 0};
+    for (int s = count - 1; s >= 0; s--) {
+        if (s < count - 1) {
+            const double *r = rec + (size_t)s * kAdjRec;
+            const double *rn = r + kAdjRec;
+            const double h = __ldg(r + 1) - __ldg(r), ih = 1.0 / h, h2 = h * h;
+            double phi[9][3], u[9][3], add[3];
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                const double lvh = lv[c] * ih;
+#pragma unroll
+                for (int k = 0; k < 9; k++)
+                    phi[k][c] = fma(g_adj.W2f[8][k], lx[c], g_adj.W1f[8][k] * lvh);
+                lv[c] = fma(h, lx[c], lv[c]);
+                add[c] = 0.0;
+            }
+            // midpoints inside the step
+            for (; kb >= 0 && bidx[kb] == s && bfrac[kb] != 0.0; kb--) {
+                const double *g = gjump + kb * 6;
+                const double f = bfrac[kb];
+                double gx[3], gv[3];
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    gx[c] = g[c];
+                    gv[c] = g[3 + c];
+                    add[c] += gx[c];
+                    lv[c] += fma(f * h, gx[c], gv[c]);
+                    gx[c] *= f * f;
+                    gv[c] *= f * ih;
+                }
+#pragma unroll
+                for (int k = 0; k < 9; k++) {   // integrals of sample k's basis to f
+                    double p2 = 0.0, p1 = 0.0;
+#pragma unroll
+                    for (int p = 8; p >= 0; p--) {
+                        p2 = fma(p2, f, g_adj.Lf[k][p] * (1.0 / ((p + 1.0) * (p + 2.0))));
+                        p1 = fma(p1, f, g_adj.Lf[k][p] * (1.0 / (p + 1.0)));
+                    }
+#pragma unroll
+                    for (int c = 0; c < 3; c++) phi[k][c] = fma(p2, gx[c], fma(p1, gv[c], phi[k][c]));
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 9; k++) {
+                jmul(jac_sample_fwd(r, rn, k), phi[k], u[k]);
+#pragma unroll
+                for (int c = 0; c < 3; c++) u[k][c] *= h2;
+            }
+            double before = 0.0, sum[3] = {0.0, 0.0, 0.0};
+            for (int it = 0; it < 12; it++) {
+                double delta = 0.0, size = 0.0, now[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+                for (int k = 8; k >= 0; k--) {
+                    double z[3];
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+                        z[c] = phi[k][c];
+#pragma unroll
+                        for (int n = 1; n < 9; n++) z[c] = fma(g_adj.W2f[n][k], u[n][c], z[c]);
+                    }
+                    jmul(jac_sample_fwd(r, rn, k), z, u[k]);
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+                        u[k][c] *= h2;
+                        now[c] += u[k][c];
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    delta = fmax(delta, fabs(now[c] - sum[c]));
+                    size = fmax(size, fabs(lx[c] + add[c] + now[c]));
+                    sum[c] = now[c];
+                }
+                // the change left before the first sweep is not a sweep's
+                if (it > 0 ? colloc_done(delta, size, before) : delta == 0.0) break;
+                if (it == 0) before = delta;
+            }
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                double acc = 0.0;
+#pragma unroll
+                for (int k = 1; k < 9; k++) acc = fma(g_adj.sigf[k], u[k][c], acc);
+                lx[c] += add[c] + sum[c];
+                lv[c] = fma(h, acc, lv[c]);
+            }
+        }
+        // midpoints at the step's start (or at the final state)
+        for (; kb >= 0 && bidx[kb] == s; kb--) {
             const double *g = gjump + kb * 6;
 #pragma unroll
             for (int c = 0; c < 3; c++) {
-                mud[c] -= g[c];       // lambda_x += dL/dx
-                mu[c] += g[3 + c];    // lambda_v += dL/dv
+                lx[c] += g[c];
+                lv[c] += g[3 + c];
             }
-            kb--;
-        }
-        if (s < 0) break;
-        if (mu[0] == 0.0 && mu[1] == 0.0 && mu[2] == 0.0 && mud[0] == 0.0 && mud[1] == 0.0 &&
-            mud[2] == 0.0)
-            continue;
-        const double *r = rec + (size_t)s * kAdjRec;
-        const double *rn = r + kAdjRec;
-        const double h = __ldg(r + 1) - __ldg(r);
-        const double h2 = h * h;
-        // s-derivative at the step end: d mu / ds = -h d mu / dt
-        const double q0[3] = {-h * mud[0], -h * mud[1], -h * mud[2]};
-        double Fk[9][3], m8[3];
-#pragma unroll
-        for (int k = 0; k < 9; k++) {
-            double mk[3];
-#pragma unroll
-            for (int c = 0; c < 3; c++) mk[c] = fma(g_adj.sig[k], q0[c], mu[c]);
-            jmul(jac_sample(r, rn, k), mk, Fk[k]);
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                Fk[k][c] *= h2;
-                m8[c] = mk[c];
-            }
-        }
-        // Gauss-Seidel sweeps of the collocation equations (a linear system with
-        // contraction ~ h^2 |J|); at most 12
-        double before = 0.0;
-        for (int it = 0; it < 12; it++) {
-            double delta = 0.0, size = 0.0;
-#pragma unroll
-            for (int k = 1; k < 9; k++) {
-                double nm[3];
-#pragma unroll
-                for (int c = 0; c < 3; c++) {
-                    double acc = fma(g_adj.sig[k], q0[c], mu[c]);
-#pragma unroll
-                    for (int j = 0; j < 9; j++) acc = fma(g_adj.W2[k][j], Fk[j][c], acc);
-                    nm[c] = acc;
-                }
-                if (k == 8) {
-#pragma unroll
-                    for (int c = 0; c < 3; c++) {
-                        delta = fmax(delta, fabs(nm[c] - m8[c]));
-                        size = fmax(size, fabs(nm[c]));
-                        m8[c] = nm[c];
-                    }
-                }
-                jmul(jac_sample(r, rn, k), nm, Fk[k]);
-#pragma unroll
-                for (int c = 0; c < 3; c++) Fk[k][c] *= h2;
-            }
-            if (colloc_done(delta, size, before)) break;
-        }
-        double q8[3];
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            double acc = q0[c];
-#pragma unroll
-            for (int j = 0; j < 9; j++) acc = fma(g_adj.W1[8][j], Fk[j][c], acc);
-            q8[c] = acc;
-            mu[c] = m8[c];
-            mud[c] = -q8[c] / h;
         }
     }
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-        P.grad[c * P.n + gi] = -mud[c];
-        P.grad[(3 + c) * P.n + gi] = mu[c];
+        P.grad[c * P.n + gi] = lx[c];
+        P.grad[(3 + c) * P.n + gi] = lv[c];
     }
 }
 
 // ---------------------------------------------------------------------------
 // state-transition matrix at the batch midpoints
 // ---------------------------------------------------------------------------
-// sample k of a step in the forward order: J at node k (k <= 7), at the step
-// end (k = 8: the next record's node 0)
-__device__ __forceinline__ const double *jac_sample_fwd(const double *r, const double *r_next, int k)
-{
-    return k == 8 ? r_next + 2 : r + 2 + 6 * k;
-}
-
 // column c of Phi at (dx, dv), row-major 6x6 per batch
 __device__ __forceinline__ void store_column(double *ph, int c, const double dx[3], const double dv[3])
 {
@@ -1180,28 +1219,6 @@ k_adj_stm(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
     }
 }
 
-// dL/dy0 = sum over the batches of Phi^T dL/dy(t_ref): the gradient of few
-// bodies, whose state-transition matrices take six threads each where the
-// backward pass would run one lane.  Thread per body and component.
-__global__ void __launch_bounds__(128)
-k_adj_grad_phi(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
-{
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t i = idx / 6;
-    const int c = (int)(idx % 6);
-    if (i >= nc) return;
-    double g = 0.0;
-    if (B.status[i] != KETE_BODY_OK) g = __longlong_as_double(0x7ff8000000000000ll);
-    else
-        for (int k = B.nbat[i] - 1; k >= 0; k--) {
-            const double *phi = B.phi + ((size_t)i * P.m + k) * 36;
-            const double *j = B.gjump + ((size_t)i * P.m + k) * 6;
-#pragma unroll
-            for (int r = 0; r < 6; r++) g = fma(j[r], phi[6 * r + c], g);
-        }
-    P.grad[c * P.n + i0 + i] = g;
-}
-
 // ---------------------------------------------------------------------------
 // the full force model: da/dx beyond the Newtonian part and da/dv
 // ---------------------------------------------------------------------------
@@ -1264,7 +1281,7 @@ __device__ __forceinline__ void var_rhs_full(const double *J, const double *X, d
 //   mu(sig_n) = mu_0 + sig_n h lx_0 + sum_k (W2[n][k] G_k + W1[n][k] H_k),
 //   lx(1)     = lx_0 + (1/h) sum_k W1[8][k] G_k,
 // solved by Gauss-Seidel sweeps over the samples (contraction ~ h^2 |Ax| +
-// h |Av|, at most 16 sweeps).  Without the extension this is k_adj_backward.
+// h |Av|, at most 16 sweeps).  Its steps end at the batch midpoints.
 __global__ void __launch_bounds__(128)
 k_adj_backward_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 {
@@ -1522,13 +1539,6 @@ cudaError_t launch_adjoint_stm(const AdjBuffers &B, const AdjProblem &P, int64_t
     const int stm_block = nc < 4096 ? 32 : 128;   // few bodies: one warp to a block, spread over the SMs
     if (B.recx) k_adj_stm_full<<<blocks_for(6 * nc, stm_block), stm_block, 0, st>>>(B, P, i0, nc);
     else k_adj_stm<<<blocks_for(6 * nc, stm_block), stm_block, 0, st>>>(B, P, i0, nc);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_adjoint_grad_phi(const AdjBuffers &B, const AdjProblem &P, int64_t i0,
-                                    int64_t nc, cudaStream_t st)
-{
-    if (nc > 0) k_adj_grad_phi<<<blocks_for(6 * nc, 128), 128, 0, st>>>(B, P, i0, nc);
     return cudaGetLastError();
 }
 

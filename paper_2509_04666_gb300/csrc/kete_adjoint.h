@@ -50,7 +50,7 @@ struct AdjBuffers {
                        // its records carry recx; 0: a body without terms, Newtonian
                        // records only
     int32_t *status;   // [nc]
-    double *bfrac;     // [nc][m] (with phi) where in step bidx[k] batch k's midpoint
+    double *bfrac;     // [nc][m] where in step bidx[k] batch k's midpoint
                        // lies, (t_ref - t_start) / h; 0: at the step's start
     double *planets;   // [7 n_bodies 6][lanes of the forward grid]: see attempt_sweep
 };
@@ -83,10 +83,9 @@ __device__ __forceinline__ int next_batch(const kete_obs *o, int mi, int j0, dou
 }
 
 cudaError_t upload_adjoint_tables(cudaStream_t st);
-// kete_warp.cu: the forward pass with one warp per body, for few bodies without
-// non-gravitational terms: steps of
-// the size the step control proposes, the batch midpoints inside them from the
-// step polynomial (B.bfrac)
+// kete_warp.cu: the forward pass with one warp per body, without
+// non-gravitational terms: steps of the size the step control proposes, the
+// batch midpoints inside them from the step polynomial (B.bfrac)
 cudaError_t launch_adjoint_forward_warp(const EphemDev &E, const ForceDev &F, const WarpModel &W,
                                         const AdjBuffers &B, const AdjProblem &P, int64_t i0,
                                         int64_t nc, cudaStream_t st);
@@ -102,9 +101,6 @@ cudaError_t launch_adjoint_last_epoch(const AdjProblem &P, int64_t i0, int64_t n
 cudaError_t launch_adjoint_observe(const EphemDev &E, const AdjBuffers &B, const AdjProblem &P,
                                    int64_t i0, int64_t nc, cudaStream_t st);
 cudaError_t launch_adjoint_backward(const AdjBuffers &B, const AdjProblem &P, int64_t i0,
-                                    int64_t nc, cudaStream_t st);
-// the gradient from the state-transition matrices (B.phi) and B.gjump
-cudaError_t launch_adjoint_grad_phi(const AdjBuffers &B, const AdjProblem &P, int64_t i0,
                                     int64_t nc, cudaStream_t st);
 // the state-transition matrix at every batch midpoint (B.phi), integrated
 // forward over the recorded steps
