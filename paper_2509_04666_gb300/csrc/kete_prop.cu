@@ -101,7 +101,8 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
     int status = KETE_BODY_OK;
     long long attempts = 0, body_attempts = 0;
     StepState S;
-    S.have_a0 = false;
+    S.have_a0 = S.chained = false;
+    S.start = START_A0;
     S.ng = nullptr;
     S.ng_chi = 0.0;
     bool plain = true, careful = false;   // steps end at the stops; for good after a failure
@@ -144,11 +145,16 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                         }
                         t = A.t_new;
                         S.have_a0 = false;
+                        S.chained = true;
+                    } else {
+                        S.start = MODE == KETE_MIXED ? START_A0 : START_RETRY;
                     }
                 }
                 if (status != KETE_BODY_OK && !plain && k < n_stops && stops[k] != A.t_new) {
                     careful = plain = true;   // a step past a stop failed: plain steps from here
                     status = KETE_BODY_OK;
+                    S.start = START_A0;       // (its polynomial is of no use)
+                    S.chained = false;
                 }
             }
             // lanes without a body take the next ones; a body may already be
@@ -182,6 +188,7 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                             attempts = 0;
                             body_attempts = 0;
                             S.have_a0 = false;
+                            S.chained = false;
                             S.ng = (NG && F.nongrav) ? F.nongrav + i : nullptr;
                             S.ng_chi = 0.0;
                             plain = true;

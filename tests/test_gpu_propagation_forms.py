@@ -172,3 +172,27 @@ def test_target_far_off_the_table(K, pop, target):
         for i in range(20):
             rc, ref, _ = orc.propagate_stops(orc.force_model(), states[:, i], W.T0, [W.T0 + 1.0])
             assert rc == 0 and np.abs(out[0, :3, i] - ref[0, :3]).max() < TOL
+
+
+@pytest.mark.parametrize("form", ["warp", "lane", "aside"])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_rejected_steps(K, pop, form, precision):
+    """A first step far too long: its rejected polynomial, cut to the new
+    length, starts the retry; forward and backward from the same start."""
+    from paper_2509_04666_gb300 import kete
+    w, states = pop
+    states = states[:, :17]            # main belt
+    epochs = np.full(17, W.T0 + 20.0)
+    K.load_ephem(w.ephem.to_bytes())
+    _form(K, form, precision)
+    fm = kete.force_model(precision=precision, dt_init=120.0)
+    orc = O.Oracle(w.ephem.to_bytes())
+    for target in (W.T0 + 300.0, W.T0 - 40.0):
+        st, ep = _dev(states), _dev(epochs)
+        status = K.propagate(st, ep, target, fm=fm)
+        assert (status.cpu().numpy() == 0).all()
+        assert K.get_stats()["rejected"] >= (17 if target > W.T0 else 0)
+        got = st.cpu().numpy()
+        for i in range(17):
+            rc, ref, *_ = orc.propagate(orc.force_model(), states[:, i], epochs[i], target)
+            assert rc == 0 and np.abs(got[:3, i] - ref[:3]).max() < TOL, (i, form, target)
