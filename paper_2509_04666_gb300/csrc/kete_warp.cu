@@ -19,8 +19,8 @@
 //     nodes come from the Newton coefficients directly (tabulated integrals of
 //     the Newton basis), so no power-basis conversion is done.
 // About 170 FP64 instructions a sweep, 180 for the planets of an attempt and 85
-// to continue the previous step's polynomial (2.0-2.3 sweeps a step; from the
-// two-body derivatives 3.3: 1,000 comet clones over 8 years 26.5 ms, now 21.5).
+// to continue the previous step's polynomial (2.0-2.3 sweeps a step; 1,000
+// comet clones over 8 years 21.5 ms, 26.5 from the two-body derivatives).
 // Steps end only at the last stop of a direction; the stops inside a step come
 // from its polynomial, eight at a time (one per node group).
 #include <cuda_runtime.h>
