@@ -473,30 +473,33 @@ static int cost_order(kete_ctx *ctx, const double *states, int64_t stride, const
     return KETE_OK;
 }
 
-// Whether a call takes one warp per body throughout.  Measured in FP64: a step
-// takes a lane 0.45 ms and the full lane grid 0.025 us, a warp 0.03 ms and the
-// full grid of warps 0.065 us; the lane launch's last warps add 6-10 ms.  So
-// warps win below about 7,000 bodies, and on short spans as long as the extra
-// throughput of lanes does not pay for those last warps (12,000 bodies over a
-// year: 21 ms against 35; 30,000 over 120 days: 19 against 16.5; 757,000 over
-// 60 days: 260 against 104).  The steps of a body are taken as 3 to start plus
-// one in 14 days.  Mixed precision: lanes are about twice as fast.
-constexpr int64_t kWarpBodies = 8192;
+// Whether a call takes one warp per body throughout.  A step takes a lane 0.4
+// ms and the full lane grid 0.016 us, a warp 0.025 ms and the full grid of warps
+// 0.06 us, and the lanes wait for their last warps.  Measured (ms, warps /
+// lanes), catalogue bodies: 10 days 30,000 3.2 / 3.7, 60,000 6.0 / 4.2; 30 days
+// 20,000 3.7 / 4.3, 30,000 5.7 / 4.7; 90 days 12,000 6.1 / 6.7, 20,000 8.5 / 7.3;
+// a year 12,000 17.9 / 19.2, 20,000 25.6 / 19.4; mixed precision (lanes faster):
+// 10 days 20,000 2.2 / 2.6, 30,000 3.2 / 2.9; a year 12,000 17.9 / 18.3.  The steps
+// of a body are taken as 3 to start plus one in 14 days.
 static bool takes_warps(int64_t n, double span, bool mixed)
 {
     const double steps = (double)n * (3.0 + std::fabs(span) / 14.0);
-    return n <= (mixed ? kWarpBodies / 2 : kWarpBodies) || steps <= (mixed ? 150e3 : 300e3);
+    return n <= (mixed ? 12000 : 13000) || steps <= (mixed ? 95e3 : 125e3);
 }
 
 // Bodies that need far more steps than the rest would set the time of a whole
-// launch: past this many attempts they finish with one warp each.  With several
-// bodies to a lane there is time for more (the main belt takes 24 steps a
-// year; 250,000 mixed bodies over a year, 6.4 to a lane: span / 3 days 210 ms,
-// span / 8 231; 100,003 over 180 days: 82 and 65; 30,011 over 120 days: 24 and 16).
-static int attempts_budget(const kete_ctx *ctx, int64_t n, double span)
+// launch: past this many attempts they finish with one warp each (the main belt
+// takes 24 steps a year).  The more bodies there are to a lane, and the slower
+// lanes are, the longer lanes can go on with them.  Measured (ms), attempts a
+// day beyond the first six: 250,000 mixed bodies over a year 0.3 158.0, 0.6
+// 152.5; 30,011 over 120 days 0.05 8.5, 0.1 9.6, 0.3 15.5; mixed precision: 100,003
+// over 180 days 0.05 58.2, 0.1 59.4, 0.3 73.6, 250,000 over 20 days 0.15 11.3, 0.6
+// 12.8.  Below 0.075 main-belt bodies themselves are set aside.
+static int attempts_budget(const kete_ctx *ctx, int64_t n, double span, bool mixed)
 {
-    const double load = std::min(4.0, std::max(1.0, (double)n / (512.0 * ctx->n_sm)));
-    return 6 + (int)std::min(1e6, std::fabs(span) / 10.0 * load);
+    const double load = (double)n / (512.0 * ctx->n_sm);
+    const double per_day = std::min(mixed ? 0.4 : 0.6, std::max(0.075, (mixed ? 0.05 : 0.19) * load));
+    return 6 + (int)std::min(1e6, std::fabs(span) * per_day);
 }
 
 // One propagation launch (and the set-aside bodies' second one) of the chain
@@ -514,7 +517,8 @@ static int propagate_launch(kete_ctx *ctx, const ForceDev &F, ChainState cs, dou
     if (!(grid && grid->n_len == 1 && grid->J > 1) && warp_model(ctx->E, F, defer.model)) {
         GET(S_DEFER_LIST, cs.n, defer.list);
         GET(S_DEFER_CNT, 1, defer.count);
-        defer.budget0 = var.budget > 0 ? 0 : attempts_budget(ctx, cs.n, t_end - t_start);
+        defer.budget0 = var.budget > 0 ? 0 : attempts_budget(ctx, cs.n, t_end - t_start,
+                                                                 F.precision == KETE_MIXED);
         dp = &defer;
     }
     int32_t *order = nullptr;
