@@ -63,13 +63,15 @@ struct AdjTables {
     double sigf[9];
     double W1f[9][9];
     double W2f[9][9];
-    double Lf[9][9];   // l_k(s) = sum_p Lf[k][p] s^p on the forward samples
+    // first and second integrals from 0 of l_k(s) on the forward samples:
+    // s sum_p L1f[k][p] s^p, s^2 sum_p L2f[k][p] s^p
+    double L1f[9][9], L2f[9][9];
 };
 static __constant__ AdjTables g_adj;
 
 // Lagrange-basis integrals on 9 sample points sg (see AdjTables)
 static void fill_colloc(const long double sg[9], double sig[9], double W1[9][9], double W2[9][9],
-                        double L[9][9] = nullptr)
+                        double L1[9][9] = nullptr, double L2[9][9] = nullptr)
 {
     for (int n = 0; n < 9; n++) sig[n] = (double)sg[n];
     for (int k = 0; k < 9; k++) {
@@ -84,8 +86,11 @@ static void fill_colloc(const long double sg[9], double sig[9], double W1[9][9],
             deg++;
             den *= (sg[k] - sg[j]);
         }
-        if (L)
-            for (int p = 0; p < 9; p++) L[k][p] = (double)(c[p] / den);
+        if (L1)
+            for (int p = 0; p < 9; p++) {
+                L1[k][p] = (double)(c[p] / den / (p + 1));
+                L2[k][p] = (double)(c[p] / den / ((p + 1) * (p + 2)));
+            }
         for (int n = 0; n < 9; n++) {
             long double w1 = 0.0L, w2 = 0.0L, sp = sg[n];
             for (int p = 0; p <= 8; p++) {
@@ -110,7 +115,7 @@ static void fill_adj_tables(AdjTables &T)
     fill_colloc(sg, T.sig, T.W1, T.W2);
     for (int n = 0; n <= 7; n++) sg[n] = (long double)rt.h[n];
     sg[8] = 1.0L;
-    fill_colloc(sg, T.sigf, T.W1f, T.W2f, T.Lf);
+    fill_colloc(sg, T.sigf, T.W1f, T.W2f, T.L1f, T.L2f);
 }
 
 cudaError_t upload_adjoint_tables(cudaStream_t st)
@@ -968,7 +973,7 @@ __device__ __forceinline__ bool colloc_done(double delta, double size, double &b
 //   lambda_v <- lambda_v + h lambda_x + sum (g_v + s h g_x) + h sum s_n u_n.
 // It is the exact transpose of k_adj_stm.  Gauss-Seidel sweeps from the step's
 // end (W2f is nearly lower triangular; contraction ~ h^2 |J|), at most 12.
-// FP64 issue bounds it: a sweep is 330 multiply-adds, a midpoint 400.  With the
+// FP64 issue bounds it: a sweep is 330 multiply-adds, a midpoint 220.  With the
 // forward pass stopping at no midpoint (6-7 steps instead of 25 over 90 days and
 // 20 midpoints), 100,000 bodies: loss and gradient 164 -> 68.6 ms.
 __global__ void __launch_bounds__(128)
@@ -1022,8 +1027,8 @@ k_adj_backward(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
                     double p2 = 0.0, p1 = 0.0;
 #pragma unroll
                     for (int p = 8; p >= 0; p--) {
-                        p2 = fma(p2, f, g_adj.Lf[k][p] * (1.0 / ((p + 1.0) * (p + 2.0))));
-                        p1 = fma(p1, f, g_adj.Lf[k][p] * (1.0 / (p + 1.0)));
+                        p2 = fma(p2, f, g_adj.L2f[k][p]);
+                        p1 = fma(p1, f, g_adj.L1f[k][p]);
                     }
 #pragma unroll
                     for (int c = 0; c < 3; c++) phi[k][c] = fma(p2, gx[c], fma(p1, gv[c], phi[k][c]));
@@ -1117,9 +1122,9 @@ __device__ __forceinline__ void colloc_at(const double F[9][3], double h, double
         for (int p = 8; p >= 0; p--) {
             double cp = 0.0;
 #pragma unroll
-            for (int k = 0; k < 9; k++) cp = fma(g_adj.Lf[k][p], F[k][c], cp);
-            p2 = fma(p2, s, cp * (1.0 / ((p + 1.0) * (p + 2.0))));
-            p1 = fma(p1, s, cp * (1.0 / (p + 1.0)));
+            for (int k = 0; k < 9; k++) cp = fma(g_adj.L1f[k][p], F[k][c], cp);
+            p2 = fma(p2, s, cp * (1.0 / (p + 2.0)));
+            p1 = fma(p1, s, cp);
         }
         dx[c] = fma(s * s, p2, fma(s * h, dv0[c], dx0[c]));
         dv[c] = fma(s / h, p1, dv0[c]);
