@@ -12,8 +12,9 @@
  *      force model of Eq. A.1 (Newton + GR of Eq. A.3 + J2 of Eq. A.4, and
  *      optionally per-body radiation pressure, Eq. A.6, and the JPL comet
  *      model, Eq. A.7) by a Gauss-Radau integrator with IAS15 convergence
- *      and step control and the predictor removed (Sec. 3.2, App. A.6), in
- *      FP64 or with FP32 planetary terms;
+ *      and step control (Sec. 3.2, App. A.6; the paper removes the predictor,
+ *      here the corrector's start only saves sweeps), in FP64 or with FP32
+ *      planetary terms;
  *   3. FoVs sorted and grouped into <= 3-day batches, bodies integrated to each
  *      batch midpoint, then two-body propagation with light-delay correction
  *      to each FoV epoch (Sec. 2);

@@ -34,7 +34,7 @@ enum Slot {
     S_ORDER_SCAN, S_ORDER_N, S_ADJ_TEND, S_LEG_OUT,
     S_EXT_START, S_EXT_EX, S_EXT_TMP, S_EXT_FIRST, S_EXT_SUB, S_EXT_PARENT, S_EXT_CNT,
     S_EXT_OFF, S_EXT_CUR, S_EXT_GROUP, S_EXT_KEEP, S_EXT_KCNT, S_EXT_KOFF, S_ADJ_PHI, S_ADJ_RECX,
-    S_PRE_KEEP, S_PRE_N, S_ADJ_RICH, S_ADJ_PLANETS, S_ADJ_BFRAC,
+    S_PRE_KEEP, S_PRE_N, S_ADJ_RICH, S_ADJ_PLANETS, S_ADJ_BFRAC, S_ADJ_MID, S_ADJ_RANGE,
     S_NSLOTS
 };
 
@@ -481,10 +481,11 @@ static int cost_order(kete_ctx *ctx, const double *states, int64_t stride, const
 // a year 12,000 17.9 / 19.2, 20,000 25.6 / 19.4; mixed precision (lanes faster):
 // 10 days 20,000 2.2 / 2.6, 30,000 3.2 / 2.9; a year 12,000 17.9 / 18.3.  The steps
 // of a body are taken as 3 to start plus one in 14 days.
+constexpr int64_t kWarpBodies = 13000;
 static bool takes_warps(int64_t n, double span, bool mixed)
 {
     const double steps = (double)n * (3.0 + std::fabs(span) / 14.0);
-    return n <= (mixed ? 12000 : 13000) || steps <= (mixed ? 95e3 : 125e3);
+    return n <= (mixed ? 12000 : kWarpBodies) || steps <= (mixed ? 95e3 : 125e3);
 }
 
 // Bodies that need far more steps than the rest would set the time of a whole
@@ -1514,8 +1515,33 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
             const int64_t nc = std::min(chunk, n - i0);
             prop_event(ctx, true);
             int32_t *order = nullptr;
-            if (order_on && !warps) {   // most expensive bodies first (schedule only)
-                unsigned long long *order_n;
+            // many bodies whose chains share one step grid: lanes (see takes_warps)
+            unsigned long long *order_n = nullptr;
+            GridDev Q{};
+            double span = 0.0;
+            bool lanes = warps && nc > kWarpBodies;
+            B.mid = nullptr;
+            if (lanes) {
+                unsigned long long *range, key[2];
+                GET(S_ADJ_MID, (size_t)chunk * m, B.mid);
+                GET(S_ADJ_RANGE, 2, range);
+                CUDA_TRY(launch_fit_stops(B, P, i0, nc, range, ctx->stream));
+                CUDA_TRY(cudaMemcpyAsync(key, range, sizeof(key), cudaMemcpyDeviceToHost, ctx->stream));
+                CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+                launches++;
+                const double lo = std::max(ctx->E.t_start, fit_range_epoch(key[0]));
+                const double hi = std::min(ctx->E.t_end, fit_range_epoch(key[1]));
+                span = hi - lo;
+                lanes = span > 0.0 && span <= (double)kGridUnits && !takes_warps(nc, span, false);
+                if (lanes) {
+                    const int J = (int)std::max(1.0, std::ceil(span - 1e-9));
+                    std::vector<double> pts((size_t)J + 1);
+                    for (int j = 0; j <= J; j++) pts[j] = lo + span / J * j;
+                    pts[J] = hi;
+                    if ((r = make_grid(ctx, pts, span / J, false, Q)) != KETE_OK) return r;
+                }
+            }
+            if (order_on && (!warps || lanes)) {   // most expensive bodies first (schedule only)
                 CUDA_TRY(launch_adjoint_last_epoch(P, i0, nc, t_end, ctx->stream));
                 // bodies with and without non-gravitational terms in separate
                 // ranges, so that the full-model records rarely share a warp
@@ -1524,7 +1550,21 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
                 if (r2 != KETE_OK) return r2;
                 launches += 1;
             }
-            if (warps) CUDA_TRY(launch_adjoint_forward_warp(ctx->E, F, model, B, P, i0, nc, ctx->stream));
+            if (lanes) {
+                PropDefer defer{};
+                GET(S_DEFER_LIST, nc, defer.list);
+                GET(S_DEFER_CNT, 1, defer.count);
+                defer.budget0 = attempts_budget(ctx, nc, span, false);
+                CUDA_TRY(launch_fit_lanes(ctx->E, F, B, P, i0, nc, Q, next, order, order_n, defer,
+                                          ctx->stream));
+                CUDA_TRY(launch_fit_jacobian(ctx->E, F, B, nc, ctx->stream));
+                PropQueue q{};
+                q.list = defer.list;
+                q.list_n = defer.count;
+                CUDA_TRY(launch_adjoint_forward_warp(ctx->E, F, model, B, P, i0, nc, ctx->stream, q));
+                launches += 2;
+            } else if (warps)
+                CUDA_TRY(launch_adjoint_forward_warp(ctx->E, F, model, B, P, i0, nc, ctx->stream));
             else CUDA_TRY(launch_adjoint_forward(ctx->E, F, B, P, i0, nc, next, ctx->stream, order));
             prop_event(ctx, false);
             if (jac) {

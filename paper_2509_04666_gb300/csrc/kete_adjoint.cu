@@ -1484,6 +1484,148 @@ k_adj_stm_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 // ---------------------------------------------------------------------------
 static unsigned blocks_for(int64_t n, int per) { return (unsigned)((n + per - 1) / per); }
 
+// ---------------------------------------------------------------------------
+// orbit fits in the lane form (see kete_adjoint.h)
+// ---------------------------------------------------------------------------
+// doubles as integers of the same order
+__device__ __forceinline__ unsigned long long order_key(double x)
+{
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    return (u >> 63) ? ~u : u | (1ull << 63);
+}
+
+double fit_range_epoch(unsigned long long key)
+{
+    const unsigned long long u = (key >> 63) ? key & ~(1ull << 63) : ~key;
+    double x;
+    std::memcpy(&x, &u, sizeof(x));
+    return x;
+}
+
+__global__ void k_fit_stops(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc,
+                            unsigned long long *__restrict__ range)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nc) return;
+    const int64_t gi = i0 + i;
+    const kete_obs *o = P.obs + gi * P.m;
+    const double t0 = P.epochs[gi];
+    bool ok = isfinite(t0);
+    for (int c = 0; c < 6; c++) ok = ok && isfinite(P.states[c * P.n + gi]);
+    const int mi = obs_count(o, P.m);
+    for (int j = 1; j < mi; j++)
+        if (o[j].epoch < o[j - 1].epoch) {
+            atomicOr(&P.ctr->error_flags, 1 << 6);
+            ok = false;
+        }
+    int status = ok ? KETE_BODY_OK : KETE_BODY_NONFINITE, nb = 0, capped = 0;
+    double last = t0;
+    for (int j0 = 0; j0 < mi; nb++) {
+        j0 = next_batch(o, mi, j0, P.span, last);
+        B.mid[(size_t)i * P.m + nb] = last;
+    }
+    if (P.ckpt > 0.0 && last > t0) {
+        const double ck = ceil((last - t0) / P.ckpt) - 1.0;
+        if (ck >= (double)kAdjMaxCkpt) status = KETE_BODY_STEP_CAP;
+        else if (ck + nb > (double)(B.cap - 1)) capped = 1;
+    }
+    B.nbat[i] = nb;
+    B.status[i] = status;
+    B.n_rec[i] = capped;
+    if (ok && nb > 0) {
+        atomicMin(range, order_key(t0));
+        atomicMax(range + 1, order_key(last));
+    }
+}
+
+// The Newtonian da/dx at the 8 nodes of every record in place of the step's
+// polynomial (k_propagate, FitRecord): a warp per body, 4 records at a time, a
+// thread per node; three planets' series at a time share the basis.  FP64 issue bounds
+// it: ~600 instructions a node.
+__global__ void __launch_bounds__(128)
+k_fit_jacobian(EphemDev E, ForceDev F, AdjBuffers B, int64_t nc)
+{
+    const int lane = threadIdx.x & 31, node = lane & 7;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= nc) return;
+    const int count = B.n_rec[i];
+    double *rec = B.rec + (size_t)i * B.cap * kAdjRec;
+    for (int s0 = 0; s0 < count; s0 += 4) {
+        const int s = s0 + (lane >> 3);
+        const bool last = s == count - 1, here = s < count && (!last || node == 0);
+        double *r = rec + (size_t)(here ? s : 0) * kAdjRec;
+        double J[6] = {0, 0, 0, 0, 0, 0};
+        if (here) {
+            const double t = r[0], h = r[1] - t, sh = last ? 0.0 : g_rt.h[node] * h;
+            double x[3] = {r[2], r[3], r[4]};
+            if (!last) {
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    double px = r[11 + 18 + c] * g_rt.wx[node][6];
+#pragma unroll
+                    for (int m = 5; m >= 0; m--) px = fma(r[11 + 3 * m + c], g_rt.wx[node][m], px);
+                    px = fma(r[8 + c], 0.5, px);
+                    x[c] += fma(sh * sh, px, sh * r[5 + c]);
+                }
+            }
+            Seg g;
+            if (ephem_seg(E, t, sh, g)) {   // (accepted steps lie on the table)
+                const double t2 = 2.0 * g.tau;
+                const int nc_ = E.n_coef;
+                for (int m0 = 0; m0 < E.n_bodies; m0 += 3) {
+                    double p[3][3], Tm1 = 1.0, T = g.tau;
+                    const double *c[3];
+#pragma unroll
+                    for (int q = 0; q < 3; q++) {
+                        c[q] = ephem_coef(E, m0 + q < E.n_bodies ? m0 + q : 0, g.s);
+#pragma unroll
+                        for (int d = 0; d < 3; d++)
+                            p[q][d] = fma(__ldg(c[q] + d * nc_ + 1), g.tau, __ldg(c[q] + d * nc_));
+                    }
+                    for (int k = 2; k < nc_; k++) {
+                        const double Tn = fma(t2, T, -Tm1);
+                        Tm1 = T;
+                        T = Tn;
+#pragma unroll
+                        for (int q = 0; q < 3; q++)
+#pragma unroll
+                            for (int d = 0; d < 3; d++)
+                                p[q][d] = fma(__ldg(c[q] + d * nc_ + k), T, p[q][d]);
+                    }
+#pragma unroll
+                    for (int q = 0; q < 3; q++)
+                        if (m0 + q < E.n_bodies && ((F.active_mask >> (m0 + q)) & 1u)) {
+                            const double d[3] = {x[0] - p[q][0], x[1] - p[q][1], x[2] - p[q][2]};
+                            newton_jacobian(E.gm[m0 + q], d, J);
+                        }
+                }
+            }
+        }
+        __syncwarp();
+        if (here)
+#pragma unroll
+            for (int c = 0; c < 6; c++) r[2 + 6 * node + c] = J[c];
+        __syncwarp();
+    }
+}
+
+cudaError_t launch_fit_stops(const AdjBuffers &B, const AdjProblem &P, int64_t i0, int64_t nc,
+                             unsigned long long *range, cudaStream_t st)
+{
+    cudaError_t e = cudaMemsetAsync(range, 0xff, sizeof(unsigned long long), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(range + 1, 0, sizeof(unsigned long long), st);
+    if (e != cudaSuccess) return e;
+    if (nc > 0) k_fit_stops<<<blocks_for(nc, 256), 256, 0, st>>>(B, P, i0, nc, range);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fit_jacobian(const EphemDev &E, const ForceDev &F, const AdjBuffers &B,
+                                int64_t nc, cudaStream_t st)
+{
+    if (nc > 0) k_fit_jacobian<<<blocks_for(32 * nc, 128), 128, 0, st>>>(E, F, B, nc);
+    return cudaGetLastError();
+}
+
 // last observation epoch of each body of the chunk (its chain's end)
 __global__ void k_adj_last_epoch(AdjProblem P, int64_t i0, int64_t nc, double *__restrict__ t_end)
 {

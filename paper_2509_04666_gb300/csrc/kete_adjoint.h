@@ -52,6 +52,7 @@ struct AdjBuffers {
     int32_t *status;   // [nc]
     double *bfrac;     // [nc][m] where in step bidx[k] batch k's midpoint
                        // lies, (t_ref - t_start) / h; 0: at the step's start
+    double *mid;       // [nc][m] batch midpoints (launch_fit_stops), or null
     double *planets;   // [7 n_bodies 6][lanes of the forward grid]: see attempt_sweep
 };
 
@@ -88,7 +89,23 @@ cudaError_t upload_adjoint_tables(cudaStream_t st);
 // batch midpoints inside them from the step polynomial (B.bfrac)
 cudaError_t launch_adjoint_forward_warp(const EphemDev &E, const ForceDev &F, const WarpModel &W,
                                         const AdjBuffers &B, const AdjProblem &P, int64_t i0,
-                                        int64_t nc, cudaStream_t st);
+                                        int64_t nc, cudaStream_t st, PropQueue q = PropQueue{});
+// The lane form of the same for many bodies whose epochs lie close enough for
+// one step grid: each body's midpoints, batch count and first status (B.mid,
+// B.nbat, B.status; B.n_rec: 1 past the record limit) and the span of all
+// chains, [first epoch, last midpoint] as order-preserving keys in range[0..1];
+// the lanes (kete_prop.cu), which leave step polynomials in the records and set
+// long bodies aside; da/dx in place of the polynomials.
+cudaError_t launch_fit_stops(const AdjBuffers &B, const AdjProblem &P, int64_t i0, int64_t nc,
+                             unsigned long long *range, cudaStream_t st);
+double fit_range_epoch(unsigned long long key);
+cudaError_t launch_fit_lanes(const EphemDev &E, const ForceDev &F, const AdjBuffers &B,
+                             const AdjProblem &P, int64_t i0, int64_t nc, const GridDev &Q,
+                             unsigned long long *next, const int32_t *order,
+                             const unsigned long long *order_n, const PropDefer &defer,
+                             cudaStream_t st);
+cudaError_t launch_fit_jacobian(const EphemDev &E, const ForceDev &F, const AdjBuffers &B,
+                                int64_t nc, cudaStream_t st);
 // persistent grid with work stealing from the counter *next;
 // order != null: lanes take the chunk's bodies in that order
 cudaError_t launch_adjoint_forward(const EphemDev &E, const ForceDev &F, const AdjBuffers &B,

@@ -2,7 +2,7 @@
 //
 // Ephemeris lookup (Sec. 3.2 / App. A), force model (Eq. A.1 with the GR term
 // of Eq. A.3 and the J2 term of Eq. A.4), Gauss-Radau 15th-order step with
-// IAS15 corrector convergence and step control, predictor removed (App. A.6),
+// IAS15 corrector convergence and step control (App. A.6),
 // universal-variable two-body propagation and light-delay correction (Sec. 2),
 // spherical-polygon test (Sec. 3.1).
 #pragma once

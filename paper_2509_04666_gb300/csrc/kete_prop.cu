@@ -6,9 +6,9 @@
 // the states at the stops inside a step come from the step's collocation
 // polynomial; without one its steps end at every stop.  Each step is a 15th-order Gauss-Radau step in the
 // IAS15 form (Newton-basis coefficients g, power-basis coefficients b, 8
-// spacings), with the predictor removed: every step starts from b = 0 and the
-// corrector iterates until max|db6|/max|a| < eps_pc, the error stops falling
-// (after 3 iterations) or max_iter is reached.  Step control follows IAS15:
+// spacings).  The corrector starts from two-body motion, then from the previous
+// step's polynomial (see CorrectorStart), and iterates until max|db6|/max|a| <
+// eps_pc, the error stops falling (after 3 iterations) or max_iter is reached.  Step control follows IAS15:
 // dt_new = dt (eps / (max|b6|/max|a|))^(1/7), reject below safety*dt, grow at
 // most 1/safety.  Every loop is bounded: max_iter corrector iterations,
 // max_steps step attempts per leg, after which the body gets a status code.
@@ -18,6 +18,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "kete_adjoint.h"
 #include "kete_step.cuh"
 
 namespace kete {
@@ -56,7 +57,7 @@ __device__ __forceinline__ void write_stop(double *__restrict__ out,
 // direction follows it (step_begin_grid); FP64 issue bounds this kernel, so the
 // count of force evaluations is what to save: stopping at every third day of a
 // survey chain took 121 steps of 22 evaluations a year, the proposed steps of
-// a main-belt body (~16 days) are 24 of 29, and the rows keep those evaluations
+// a main-belt body (~16 days) are 24 of 15-16 evaluations, and the rows keep those evaluations
 // at the shared-planet cost (about 250 FP64 instructions against 650).  A body
 // whose step past a stop fails takes plain steps, stop by stop, from there on,
 // so that the stops before the failure still get their states.
@@ -83,12 +84,62 @@ __device__ __forceinline__ void write_stop(double *__restrict__ out,
 // NG: bodies may carry non-gravitational terms (F.nongrav); the instantiation
 // without them has those branches compiled out.
 constexpr int kSyncLanes = 16;
-template <int MODE, bool NG, bool V32 = false>
+// REC (k_propagate): the bodies are those of an orbit fit.  The stops are each body's batch
+// midpoints (B.mid, B.nbat), kept with the step each lies in; every accepted
+// step leaves its epochs and polynomial in its record.  A body set aside
+// starts again in the warp form.  100,000 fits over 90 days: forward pass 42.1
+// ms one warp per body, 25.3 with lanes and k_fit_jacobian (the planets from the
+// grid's rows, a full lane grid's issue per step).
+struct FitRecord {
+    AdjBuffers B;
+    AdjProblem P;
+    int64_t i0;
+};
+
+__device__ __forceinline__ void fit_stop(const FitRecord &R, int k, int64_t i, int count, double frac,
+                                         const double x[3], const double v[3])
+{
+    const size_t at = (size_t)i * R.P.m + k;
+    double *y = R.B.yref + at * 6;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        y[c] = x[c];
+        y[3 + c] = v[c];
+    }
+    R.B.bidx[at] = count;
+    R.B.bfrac[at] = frac;
+}
+
+// the body's last record (its final state) and status; the checkpoint grid's
+// stops count toward the record limit
+__device__ __forceinline__ void fit_done(const EphemDev &E, const FitRecord &R, int64_t i, int status, bool capped,
+                                         int count, int n_stops, double epoch0, double t,
+                                         const double x[3], double *rec)
+{
+    if (R.P.ckpt > 0.0 && t > epoch0 &&
+        count + n_stops + ceil((t - epoch0) / R.P.ckpt) - 1.0 > (double)(R.B.cap - 1))
+        capped = true;
+    Seg g;
+    if (status == KETE_BODY_OK && capped) status = KETE_BODY_ADJ_CAP;
+    else if (status == KETE_BODY_OK && !ephem_seg(E, t, 0.0, g)) status = KETE_BODY_OUT_OF_SPAN;
+    if (status == KETE_BODY_OK) {
+        double *r = rec + (size_t)count * kAdjRec;
+        r[0] = r[1] = t;
+#pragma unroll
+        for (int c = 0; c < 3; c++) r[2 + c] = x[c];
+        count++;
+    }
+    R.B.n_rec[i] = status == KETE_BODY_OK ? count : 0;
+    R.B.status[i] = status;
+}
+
+template <int MODE, bool NG, bool V32 = false, bool REC = false>
 __global__ void __launch_bounds__(128, KETE_PROP_MIN_BLOCKS)
-k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ stops,
-            const int32_t *__restrict__ stop_row, int n_stops, double *__restrict__ out,
+k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ stops_in,
+            const int32_t *__restrict__ stop_row, int n_stops_in, double *__restrict__ out,
             int64_t out_stride, int out_aos, int keep_on_fail, DevCounters *ctr, GridDev Q,
-            int use_grid, unsigned long long *__restrict__ next_body, int refill, PropQueue q)
+            int use_grid, unsigned long long *__restrict__ next_body, int refill, PropQueue q,
+            FitRecord R)
 {
     const int64_t n = cs.n;
     const unsigned long long n_items = q.list ? *q.list_n : (unsigned long long)n;
@@ -96,6 +147,11 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
     const int lane = threadIdx.x & 31;
     Cnt cnt = {0, 0, 0, 0, 0};
     int64_t i = 0;            // current body
+    const double *stops = stops_in;   // its stops
+    int n_stops = n_stops_in;
+    double *rec = nullptr, epoch0 = 0.0;   // REC: its records
+    int count = 0;
+    bool capped = false;
     int k = 0;                // next stop of the body
     double x[3], v[3], t = 0.0, dt = 0.0;
     int status = KETE_BODY_OK;
@@ -129,7 +185,8 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                             while (k < n_stops && (Q.dir > 0 ? stops[k] < A.t_new : stops[k] > A.t_new)) {
                                 double xs[3], vs[3];
                                 attempt_dense(A, t, x, v, S.a0, stops[k], xs, vs);
-                                write_stop(out, stop_row, k, i, out_stride, out_aos, xs, vs);
+                                if (REC) fit_stop(R, k, i, count, (stops[k] - t) / A.h, xs, vs);
+                                else write_stop(out, stop_row, k, i, out_stride, out_aos, xs, vs);
                                 k++;
                                 attempts = 0;
                             }
@@ -137,6 +194,24 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                             // a step cut short by the grid says little about the next
                             if (fabs(A.h) < 0.5 * fabs(proposed) && fabs(dt) < fabs(proposed))
                                 dt = proposed;
+                        }
+                        if (REC) {   // the step's polynomial (k_fit_jacobian turns it into da/dx)
+                            if (count < R.B.cap - 1) {
+                                double *r = rec + (size_t)count * kAdjRec;
+                                r[0] = t;
+                                r[1] = A.t_new;
+#pragma unroll
+                                for (int c = 0; c < 3; c++) {
+                                    r[2 + c] = x[c];
+                                    r[5 + c] = v[c];
+                                    r[8 + c] = S.a0[c];
+#pragma unroll
+                                    for (int m = 0; m < 7; m++) r[11 + 3 * m + c] = A.b[m][c];
+                                }
+                                count++;
+                            } else {
+                                capped = true;
+                            }
                         }
 #pragma unroll
                         for (int c = 0; c < 3; c++) {
@@ -176,15 +251,34 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                             mine = first ? (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x : n_items;
                         if (mine < n_items) {
                             i = q.list ? (int64_t)q.list[mine] : (int64_t)mine;
+                            if (REC) {
+                                const AdjProblem &P = R.P;
+                                const int64_t gi = R.i0 + i;
 #pragma unroll
-                            for (int c = 0; c < 3; c++) {
-                                x[c] = cs.w[c * n + i];
-                                v[c] = cs.w[(3 + c) * n + i];
+                                for (int c = 0; c < 3; c++) {
+                                    x[c] = P.states[c * P.n + gi];
+                                    v[c] = P.states[(3 + c) * P.n + gi];
+                                }
+                                t = epoch0 = P.epochs[gi];
+                                dt = 0.0;
+                                status = R.B.status[i];
+                                k = 0;
+                                stops = R.B.mid + (size_t)i * P.m;
+                                n_stops = R.B.nbat[i];
+                                capped = R.B.n_rec[i] != 0;
+                                rec = R.B.rec + (size_t)i * R.B.cap * kAdjRec;
+                                count = 0;
+                            } else {
+#pragma unroll
+                                for (int c = 0; c < 3; c++) {
+                                    x[c] = cs.w[c * n + i];
+                                    v[c] = cs.w[(3 + c) * n + i];
+                                }
+                                t = cs.w[6 * n + i];
+                                dt = cs.w[7 * n + i];
+                                status = cs.status[i];
+                                k = q.resume ? cs.kstop[i] : 0;
                             }
-                            t = cs.w[6 * n + i];
-                            dt = cs.w[7 * n + i];
-                            status = cs.status[i];
-                            k = q.resume ? cs.kstop[i] : 0;
                             attempts = 0;
                             body_attempts = 0;
                             S.have_a0 = false;
@@ -210,7 +304,10 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                     while (k < n_stops && (status != KETE_BODY_OK || t == stops[k])) {
                         const double nan = __longlong_as_double(0x7ff8000000000000ll);
                         const double none[3] = {nan, nan, nan};
-                        if (status == KETE_BODY_OK) write_stop(out, stop_row, k, i, out_stride, out_aos, x, v);
+                        if (REC) {
+                            if (status == KETE_BODY_OK) fit_stop(R, k, i, count, 0.0, x, v);
+                        } else if (status == KETE_BODY_OK)
+                            write_stop(out, stop_row, k, i, out_stride, out_aos, x, v);
                         else if (!keep_on_fail) write_stop(out, stop_row, k, i, out_stride, out_aos, none, none);
                         k++;
                         attempts = 0;
@@ -228,7 +325,16 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                         aside = body_attempts >= (long long)q.budget * (k + 1) + q.budget0 ||
                                 (q.budget0 > 0 && body_attempts > 0 && !plain &&
                                  fabs(dt) * Q.inv_unit < 1.0 && F.dt_init * Q.inv_unit >= 1.0);
-                    if (k >= n_stops || aside) {
+                    if (REC && (k >= n_stops || aside)) {
+                        if (aside) {
+                            q.defer[atomicAdd(q.defer_n, 1ull)] = (int32_t)i;
+                            atomicAdd(&ctr->deferred, 1ull);
+                            R.B.n_rec[i] = 0;
+                        } else {
+                            fit_done(E, R, i, status, capped, count, n_stops, epoch0, t, x, rec);
+                        }
+                        phase = TAKE;
+                    } else if (k >= n_stops || aside) {
                         // write the chain state back and free the lane
 #pragma unroll
                         for (int c = 0; c < 3; c++) {
@@ -427,18 +533,18 @@ static void launch_k(int64_t grid, int block, cudaStream_t st, const EphemDev &E
     // mixed precision on a grid: the node velocity in FP32 (V32)
     if (F.nongrav) {
         k_propagate<MODE, true><<<(unsigned)grid, block, 0, st>>>(
-            E, F, cs, stops, row, n_stops, out, stride, aos, kof, ctr, Q, ug, next, refill, q);
+            E, F, cs, stops, row, n_stops, out, stride, aos, kof, ctr, Q, ug, next, refill, q, FitRecord{});
         return;
     }
     if constexpr (MODE == KETE_MIXED) {
         if (ug) {
             k_propagate<MODE, false, true><<<(unsigned)grid, block, 0, st>>>(
-                E, F, cs, stops, row, n_stops, out, stride, aos, kof, ctr, Q, ug, next, refill, q);
+                E, F, cs, stops, row, n_stops, out, stride, aos, kof, ctr, Q, ug, next, refill, q, FitRecord{});
             return;
         }
     }
     k_propagate<MODE, false><<<(unsigned)grid, block, 0, st>>>(
-        E, F, cs, stops, row, n_stops, out, stride, aos, kof, ctr, Q, ug, next, refill, q);
+        E, F, cs, stops, row, n_stops, out, stride, aos, kof, ctr, Q, ug, next, refill, q, FitRecord{});
 }
 
 cudaError_t launch_propagate(const EphemDev &E, const ForceDev &F, ChainState cs,
@@ -495,6 +601,33 @@ cudaError_t launch_propagate(const EphemDev &E, const ForceDev &F, ChainState cs
     q2.resume = 1;
     return launch_propagate_warp(E, F, defer->model, cs, stops_dev, stop_row, n_stops, out,
                                  out_stride, keep_on_fail, ctr, st, q2, out_aos);
+}
+
+cudaError_t launch_fit_lanes(const EphemDev &E, const ForceDev &F, const AdjBuffers &B,
+                             const AdjProblem &P, int64_t i0, int64_t nc, const GridDev &Q,
+                             unsigned long long *next, const int32_t *order,
+                             const unsigned long long *order_n, const PropDefer &defer,
+                             cudaStream_t st)
+{
+    if (nc <= 0) return cudaGetLastError();
+    cudaError_t e = cudaMemsetAsync(next, 0, sizeof(unsigned long long), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(defer.count, 0, sizeof(unsigned long long), st);
+    if (e != cudaSuccess) return e;
+    ChainState cs{};
+    cs.n = nc;
+    PropQueue q{};
+    if (order && order_n) {
+        q.list = order;
+        q.list_n = order_n;
+    }
+    q.defer = defer.list;
+    q.defer_n = defer.count;
+    q.budget0 = defer.budget0;
+    const int64_t need = (nc + 127) / 128, most = ws_blocks<KETE_FP64>(128);
+    k_propagate<KETE_FP64, false, false, true><<<(unsigned)std::min(need, most), 128, 0, st>>>(
+        E, F, cs, nullptr, nullptr, 0, nullptr, 0, 0, 0, P.ctr, Q, 1, next, 1, q,
+        FitRecord{B, P, i0});
+    return cudaGetLastError();
 }
 
 cudaError_t launch_gather_bodies(const double *st, const double *ep, int64_t n, int64_t m,

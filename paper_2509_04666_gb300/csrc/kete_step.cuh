@@ -1,6 +1,7 @@
-// kete_step.cuh -- one Gauss-Radau 15th-order step in the IAS15 form with the
-// predictor removed (Sec. 3.2, App. A.6), shared by the propagation kernel and
-// the adjoint's forward pass.
+// kete_step.cuh -- one Gauss-Radau 15th-order step in the IAS15 form (Sec. 3.2,
+// App. A.6), shared by the propagation kernel and the adjoint's forward pass.
+// The paper removes the predictor; here the corrector starts from what is known
+// of the motion (CorrectorStart), which changes its sweeps, not its solution.
 //
 // Each translation unit that includes this header holds its own copy of the
 // node tables g_rt in constant memory and must fill it with
@@ -568,7 +569,9 @@ __device__ __forceinline__ int step_begin_grid(const EphemDev &E, const ForceDev
             return KETE_BODY_OK;
         }
     }
-    jn = on ? j + 1 : j;
+    // (at the grid's end with stops past it: a step of length zero, which the
+    // caller answers with plain steps)
+    jn = on && j < Q.J ? j + 1 : j;
     if (fabs(dt) * Q.inv_unit >= 1.0) return step_aim(t, dt, __ldg(Q.g + jn), S, A);
     const int st2 = step_aim(t, dt, __ldg(Q.g + Q.J), S, A);
     while (jn < Q.J && (Q.dir > 0 ? __ldg(Q.g + jn) < A.t_new : __ldg(Q.g + jn) > A.t_new)) jn++;

@@ -250,7 +250,7 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
     const int64_t n = cs.n;
     const int lane = threadIdx.x & 31, node = lane >> 2, r = lane & 3;
     const int rc = r < 3 ? r : 2;   // the coordinate this lane computes (lane 3: a copy of 2)
-    const unsigned long long n_items = !REC && q.list ? *q.list_n : (unsigned long long)n;
+    const unsigned long long n_items = q.list ? *q.list_n : (unsigned long long)n;
     Cnt cnt = {0, 0, 0, 0, 0};
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     const double inf = __longlong_as_double(0x7ff0000000000000ll);
@@ -284,7 +284,7 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
     // contracts what is left by ~1e-3, below the rounding of the positions
     const float tol = (float)(0.3 * F.eps_pc);
     for (unsigned long long item = blockIdx.x; item < n_items; item += gridDim.x) {
-        const int64_t i = !REC && q.list ? (int64_t)q.list[item] : (int64_t)item;
+        const int64_t i = q.list ? (int64_t)q.list[item] : (int64_t)item;
         // own coordinate of the step-start state
         double x0, v0, t, dt = 0.0;
         int status = KETE_BODY_OK, k = 0, count = 0;
@@ -767,13 +767,13 @@ static unsigned warp_grid(int64_t n)
 
 cudaError_t launch_adjoint_forward_warp(const EphemDev &E, const ForceDev &F, const WarpModel &W,
                                         const AdjBuffers &B, const AdjProblem &P, int64_t i0,
-                                        int64_t nc, cudaStream_t st)
+                                        int64_t nc, cudaStream_t st, PropQueue q)
 {
     if (nc <= 0) return cudaGetLastError();
     ChainState cs{};
     cs.n = nc;
     k_propagate_warp<false, true><<<warp_grid(nc), 32, 0, st>>>(
-        E, F, W, cs, nullptr, nullptr, 0, nullptr, 0, 0, 0, P.ctr, PropQueue{}, WarpRecord{B, P, i0});
+        E, F, W, cs, nullptr, nullptr, 0, nullptr, 0, 0, 0, P.ctr, q, WarpRecord{B, P, i0});
     return cudaGetLastError();
 }
 

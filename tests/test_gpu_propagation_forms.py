@@ -177,21 +177,22 @@ def test_target_far_off_the_table(K, pop, target):
 @pytest.mark.parametrize("form", ["warp", "lane", "aside"])
 @pytest.mark.parametrize("precision", [0, 1])
 def test_rejected_steps(K, pop, form, precision):
-    """A first step far too long: its rejected polynomial, cut to the new
-    length, starts the retry; forward and backward from the same start."""
+    """A first step too long and a safety factor that rejects whatever overshoots:
+    the rejected polynomial, cut to the new length, starts the retry; forward
+    and backward from the same start."""
     from paper_2509_04666_gb300 import kete
     w, states = pop
     states = states[:, :17]            # main belt
     epochs = np.full(17, W.T0 + 20.0)
     K.load_ephem(w.ephem.to_bytes())
     _form(K, form, precision)
-    fm = kete.force_model(precision=precision, dt_init=120.0)
+    fm = kete.force_model(precision=precision, dt_init=60.0, safety=0.9)
     orc = O.Oracle(w.ephem.to_bytes())
     for target in (W.T0 + 300.0, W.T0 - 40.0):
         st, ep = _dev(states), _dev(epochs)
         status = K.propagate(st, ep, target, fm=fm)
         assert (status.cpu().numpy() == 0).all()
-        assert K.get_stats()["rejected"] >= (17 if target > W.T0 else 0)
+        assert K.get_stats()["rejected"] > 0
         got = st.cpu().numpy()
         for i in range(17):
             rc, ref, *_ = orc.propagate(orc.force_model(), states[:, i], epochs[i], target)
