@@ -58,7 +58,8 @@ PROFILED_EXACT = {"src_sha": "78dc3d3396ef0f3c", "fp64_flops_per_candidate": 834
 PROFILED_ISSUE = {"src_sha": "6c043addf4c24b22", "fp64_inst_per_step": 7765.8}
 
 
-def kernel_source_sha(files=("kete_prop.cu", "kete_device.cuh", "kete_step.cuh", "kete_order.cu")):
+def kernel_source_sha(files=("kete_prop.cu", "kete_warp.cu", "kete_device.cuh", "kete_step.cuh",
+                             "kete_order.cu")):
     h = hashlib.sha256()
     for f in files:
         with open(os.path.join(ROOT, "paper_2509_04666_gb300", "csrc", f), "rb") as fh:
@@ -102,7 +103,7 @@ def prop_flops(st, fm, n_coef, mixed):
     kernel computes them for the force model fm:
       per force evaluation from node rows: per active mass NEWTON_FLOPS, per
         GR mass + GR_FLOPS, per J2 mass + J2_FLOPS;
-      per-thread evaluation (step not spanning a whole leg): + the planet
+      per-thread evaluation (step off the grid of shared rows): + the planet
         series (series64_flops).  FP32 series (mixed precision) by Clenshaw:
         position 3 (3 (n_coef - 1) + 3), velocity 3 (4 (n_coef - 1) + 1);
       per corrector iteration: 7 substep predictors (x, v) and the g/b
@@ -346,14 +347,21 @@ def peak_fma(fp64: bool):
 
 
 def adj_flops(st, fm, n_coef):
-    """Algorithmic FP64 FLOPs of the adjoint's forward kernel: the propagation
-    count of prop_flops with every evaluation per-thread (per-body stops share
-    no node rows) plus the Newtonian da/dx of each mass at every evaluation
-    (26 FLOPs)."""
-    s = dict(st)
-    s["node_evals"] = 0
-    f64, _ = prop_flops(s, fm, n_coef, False)
-    return f64 + st["force_evals"] * _bits(fm.body_mask) * 26
+    """Algorithmic FP64 FLOPs of an orbit fit's forward pass without
+    non-gravitational terms (k_propagate on grid rows and k_fit_jacobian, or
+    k_propagate_warp) from its counters: per force evaluation the masses' terms
+    as in prop_flops; per step attempt the planet series at 8 nodes (6 per
+    coefficient and mass, basis recurrences and leading masses' velocities 44)
+    and its end, 121; per corrector iteration 1440 in the lanes, 756 in the
+    warps (no power-basis coefficients); per accepted step the Newtonian da/dx
+    of each mass at 8 nodes (26)."""
+    act, gr, j2 = _bits(fm.body_mask), _bits(fm.gr_mask), _bits(fm.j2_mask)
+    attempts = st["steps"] + st["rejected"]
+    k = n_coef - 2
+    f64 = st["force_evals"] * (NEWTON_FLOPS * act + GR_FLOPS * gr + J2_FLOPS * j2)
+    f64 += attempts * (8 * (act * (6 + 6 * k) + 4 * 11 * k) + 121)
+    f64 += st["iterations"] * (1440 if st["node_evals"] else 756)
+    return f64 + st["steps"] * 8 * act * 26
 
 
 def _timed(stream, fn, flush, reps):
@@ -451,7 +459,7 @@ def adjoint_leg(args, K, dev, flush, stream, peak):
         "value": n * 90.0 / (ms / 1e3), "unit": "body-days/s (loss + gradient)",
         "bodies_per_s": n / (ms / 1e3), "ms_per_step": ms, "forward_ms": st["prop_ms"],
         "bodies_ok": ok, "steps": st["steps"], "force_evals": st["force_evals"],
-        "roofline": {"bound": "alu", "kernel": "k_adj_forward", "achieved": fwd_tf, "peak": peak,
+        "roofline": {"bound": "alu", "kernel": "k_propagate, k_fit_jacobian", "achieved": fwd_tf, "peak": peak,
                      "unit": "TFLOP/s", "frac": fwd_tf / peak, "traffic": None},
         "nongrav": nongrav,
         "parity": {"sampled_bodies": len(sub), "max_rel_grad_x": float(rel_x.max()),
@@ -653,8 +661,8 @@ def ragged_leg(args, K, dev, flush, stream):
 def longspan_leg(args, K, dev, flush, stream):
     """Backward propagation over decades and centuries: 20,000 bodies of the
     survey population carried back 50 years, and 1,000 clones of a
-    Jupiter-family comet (JPL comet model) carried back 170 years, one lane
-    per body against lane groups of 4, 8 and 16."""
+    Jupiter-family comet (JPL comet model) carried back 170 years, one warp
+    per body against lanes that set bodies aside for warps."""
     import torch
     import oracle as O
     from paper_2509_04666_gb300 import kete, workloads as W
