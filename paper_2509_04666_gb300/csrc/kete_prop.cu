@@ -192,7 +192,10 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                             }
                             j = jn;
                             // a step cut short by the grid says little about the next
-                            if (fabs(A.h) < 0.5 * fabs(proposed) && fabs(dt) < fabs(proposed))
+                            // (its b6 is rounding, 1e-13 |a|, a growth of 3.7 at
+                            // eps 1e-9) unless its own error holds the next one back
+                            if (fabs(A.h) < 0.5 * fabs(proposed) && fabs(dt) < fabs(proposed) &&
+                                fabs(dt) >= 2.0 * fabs(A.h))
                                 dt = proposed;
                         }
                         if (REC) {   // the step's polynomial (k_fit_jacobian turns it into da/dx)
