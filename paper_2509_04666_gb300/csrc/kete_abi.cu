@@ -580,8 +580,9 @@ static int make_grid(kete_ctx *ctx, const std::vector<double> &pts, double unit,
 // t_from: the first body's epoch, or where an earlier call left the chain
 // (NaN: not known).  use_grid: follow a step grid from t_from (from the first
 // stop where t_from is not known or lies past it) in units of about a day;
-// leg_days > 0: the grid's unit, its steps of one unit only.  Marks between
-// stops far apart cut the span into launches of at most kGridUnits units.
+// leg_days > 0: the grid's unit, its steps of one unit only.  Marks (kMarkRow)
+// between stops far apart cut the span into launches of at most kGridUnits
+// units.  Grid and marks lie on the table: an epoch off it fails its own body.
 static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const double *stops,
                      int n_stops, double t_from, double *out, int64_t stride, bool keep_on_fail,
                      bool use_grid, double leg_days = 0.0, bool out_aos = false)
@@ -606,6 +607,8 @@ static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const doub
     double start = t_from;
     const double last = stops[n_stops - 1];
     if (!std::isfinite(t_from) || (last > stops[0] && t_from > stops[0])) start = stops[0];
+    const auto on_table = [&](double t) { return std::min(std::max(t, ctx->E.t_start), ctx->E.t_end); };
+    if (leg_days == 0.0) start = on_table(start);
     const bool forward = last > start;
     if (last == start) use_grid = false;
     if (leg_days == 0.0) {
@@ -620,13 +623,14 @@ static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const doub
         std::vector<int32_t> r2;
         double prev = start;
         for (int k = 0; k < n_stops; k++) {
-            const double gap = stops[k] - prev, most = unit * kGridUnits;
-            const int64_t parts = (int64_t)std::ceil(std::fabs(gap) / most);
+            const double from = leg_days > 0.0 ? prev : on_table(prev);
+            const double gap = (leg_days > 0.0 ? stops[k] : on_table(stops[k])) - from, most = unit * kGridUnits;
+            const int64_t parts = (gap > 0.0) == forward ? (int64_t)std::ceil(std::fabs(gap) / most) : 0;
             for (int64_t p = 1; p < parts; p++) {
                 // on the leg grid, where there is one
                 const double step = leg_days > 0.0 ? (gap > 0 ? most : -most) : gap / (double)parts;
-                m2.push_back(prev + step * (double)p);
-                r2.push_back(-1);
+                m2.push_back(from + step * (double)p);
+                r2.push_back(kMarkRow);
             }
             m2.push_back(stops[k]);
             r2.push_back(k);
@@ -660,7 +664,7 @@ static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const doub
             const int J = (int)std::max(1.0, std::min((double)kGridUnits, std::ceil(span / unit - 1e-9)));
             const double u = leg_days > 0.0 ? leg_days : span / J;
             std::vector<double> pts((size_t)J + 1);
-            for (int j = 0; j <= J; j++) pts[j] = start + (forward ? u : -u) * j;
+            for (int j = 0; j <= J; j++) pts[j] = start + (end > start ? u : -u) * j;
             pts[J] = end;
             const int r = make_grid(ctx, pts, u, leg_days > 0.0, Q);
             if (r != KETE_OK) return r;

@@ -77,6 +77,10 @@ struct GridDev {
     int J, n_len, nb, dir; // dir: +1 forward in time, -1 backward
     int len[kGridLens];    // step lengths in grid units, ascending from 1
 };
+// stop_row of a mark: no stop of the caller's but where a launch ends.  Bodies
+// on their way wait there for the next launch; one that starts past it (its
+// epoch is its own) stays where it is.
+constexpr int32_t kMarkRow = -2;
 
 // per-body working state of a propagation chain: [8][n] = x,y,z,vx,vy,vz,t,dt;
 // kstop[n] (may be null): the stop a set-aside body resumes at

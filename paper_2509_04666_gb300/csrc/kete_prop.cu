@@ -60,7 +60,8 @@ __device__ __forceinline__ void write_stop(double *__restrict__ out,
 // a main-belt body (~16 days) are 24 of 15-16 evaluations, and the rows keep those evaluations
 // at the shared-planet cost (about 250 FP64 instructions against 650).  A body
 // whose step past a stop fails takes plain steps, stop by stop, from there on,
-// so that the stops before the failure still get their states.
+// so that the stops before the failure still get their states.  A mark
+// (kMarkRow) ends the launch for a body on its way and none of its own.
 // A pass of the loop is one corrector sweep (7 force evaluations) for every
 // lane inside a step attempt.  An FP64 warp instruction costs the same
 // whatever its active lanes, so the work between attempts (step control, the
@@ -290,6 +291,10 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                             S.ng_chi = 0.0;
                             plain = true;
                             careful = !use_grid;
+                            if (!REC && use_grid)   // past a mark
+                                while (k < n_stops && stop_row && stop_row[k] == kMarkRow &&
+                                       (Q.dir > 0 ? t >= stops[k] : t <= stops[k]))
+                                    k++;
                             if (status == KETE_BODY_OK && k < n_stops) {
                                 aim_step(F, t, stops[k], dt);
                                 plain = careful || (stops[k] >= t) != (Q.dir > 0);
