@@ -30,7 +30,7 @@ enum Slot {
     S_HITTMP, S_FRAMECNT, S_FRAMEOFF, S_FRAMECUR, S_HITGROUP, S_MAXRAD, S_GRID, S_GRID_OK,
     S_GRID_R64, S_GRID_R32, S_STOPROW, S_XSUN, S_XOBSREL, S_NEXTBODY, S_TUNE_ST, S_TUNE_EP, S_TUNE_OUT,
     S_ADJ_REC, S_ADJ_NREC, S_ADJ_NBAT, S_ADJ_BIDX, S_ADJ_YREF, S_ADJ_GJUMP, S_ADJ_STATUS,
-    S_KSTOP, S_DEFER_LIST, S_DEFER_CNT, S_ORDER, S_ORDER_KEY, S_ORDER_HIST, S_ORDER_OFF,
+    S_KSTOP, S_TRIES, S_DEFER_LIST, S_DEFER_CNT, S_ORDER, S_ORDER_KEY, S_ORDER_HIST, S_ORDER_OFF,
     S_ORDER_SCAN, S_ORDER_N, S_ADJ_TEND, S_LEG_OUT,
     S_EXT_START, S_EXT_EX, S_EXT_TMP, S_EXT_FIRST, S_EXT_SUB, S_EXT_PARENT, S_EXT_CNT,
     S_EXT_OFF, S_EXT_CUR, S_EXT_GROUP, S_EXT_KEEP, S_EXT_KCNT, S_EXT_KOFF, S_ADJ_PHI, S_ADJ_RECX,
@@ -693,6 +693,7 @@ static int run_chain(kete_ctx *ctx, const ForceDev &F, const double *states, con
     GET(S_CHAIN, 8 * n, cs.w);
     GET(S_STATUS, n, cs.status);
     GET(S_KSTOP, n, cs.kstop);
+    GET(S_TRIES, n, cs.tries);
     cs.n = n;
     CUDA_TRY(launch_chain_init(cs, states, epochs, F, ctx->stream));
     return KETE_OK;

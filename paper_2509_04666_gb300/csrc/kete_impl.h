@@ -89,6 +89,8 @@ struct ChainState {
     int32_t *status;
     int64_t n;
     int32_t *kstop = nullptr;
+    int64_t *tries = nullptr;   // step attempts made toward the next stop (max_steps
+                                // counts them over launches; null: not kept)
 };
 
 // where a propagation launch takes its bodies from (see k_propagate)

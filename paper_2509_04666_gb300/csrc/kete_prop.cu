@@ -255,6 +255,7 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                             mine = first ? (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x : n_items;
                         if (mine < n_items) {
                             i = q.list ? (int64_t)q.list[mine] : (int64_t)mine;
+                            attempts = 0;
                             if (REC) {
                                 const AdjProblem &P = R.P;
                                 const int64_t gi = R.i0 + i;
@@ -282,8 +283,8 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                                 dt = cs.w[7 * n + i];
                                 status = cs.status[i];
                                 k = q.resume ? cs.kstop[i] : 0;
+                                if (cs.tries) attempts = cs.tries[i];
                             }
-                            attempts = 0;
                             body_attempts = 0;
                             S.have_a0 = false;
                             S.chained = false;
@@ -317,8 +318,8 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                         } else if (status == KETE_BODY_OK)
                             write_stop(out, stop_row, k, i, out_stride, out_aos, x, v);
                         else if (!keep_on_fail) write_stop(out, stop_row, k, i, out_stride, out_aos, none, none);
+                        if (!(use_grid && stop_row && stop_row[k] == kMarkRow)) attempts = 0;
                         k++;
-                        attempts = 0;
                         S.have_a0 = false;
                         if (k < n_stops && status == KETE_BODY_OK) {
                             aim_step(F, t, stops[k], dt);
@@ -352,6 +353,7 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                         cs.w[6 * n + i] = t;
                         cs.w[7 * n + i] = dt;
                         cs.status[i] = status;
+                        if (cs.tries) cs.tries[i] = attempts;
                         if (aside) {
                             cs.kstop[i] = k;
                             q.defer[atomicAdd(q.defer_n, 1ull)] = (int32_t)i;
@@ -446,6 +448,7 @@ __global__ void k_chain_init(ChainState cs, const double *__restrict__ states,
     cs.w[6 * n + i] = t;
     cs.w[7 * n + i] = 0.0;
     cs.status[i] = (ok && isfinite(t)) ? KETE_BODY_OK : KETE_BODY_NONFINITE;
+    if (cs.tries) cs.tries[i] = 0;
 }
 
 __global__ void k_chain_finish(ChainState cs, double *__restrict__ epochs,

@@ -334,7 +334,7 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
         const double epoch0 = t;
         const kete_nongrav *ng = (NG && F.nongrav) ? F.nongrav + i : nullptr;
         double ng_chi = 0.0;
-        long long attempts = 0;
+        long long attempts = !REC && cs.tries ? cs.tries[i] : 0;
         bool careful = false, have_a0 = false;
         double a0 = 0.0, bound = inf;
         double d1 = 0.0, d2 = 0.0, d3 = 0.0;   // derivatives of a at the step start
@@ -371,8 +371,8 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
                     o[r * s] = x0;
                     o[(3 + r) * s] = v0;
                 }
+                if (row != kMarkRow) attempts = 0;
                 k++;
-                attempts = 0;
                 have_a0 = false;
                 continue;
             }
@@ -746,6 +746,7 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
             cs.w[6 * n + i] = t;
             cs.w[7 * n + i] = dt;
             cs.status[i] = status;
+            if (cs.tries) cs.tries[i] = attempts;
         }
     }
     if (lane == 0) {

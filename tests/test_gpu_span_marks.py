@@ -84,3 +84,23 @@ def test_marks_move_no_body(K, pop, case, form, stops):
     assert np.nanmax(np.abs(got - ref)) < TOL
     # rounded down to the grid's lengths the lanes take more steps, not twice the way
     assert st["steps"] < 1.5 * warp["steps"] + 4 * w.n_bodies
+
+
+@pytest.mark.parametrize("form", ["warp", "lane", "aside"])
+def test_attempts_are_counted_over_the_whole_leg(K, pop, form):
+    """max_steps bounds the attempts of one leg, whatever launches it is cut into
+    and whichever form finishes it: a main-belt body makes 50 to 60 in 800 days, 30
+    or more in either half of them."""
+    from paper_2509_04666_gb300 import kete
+    w = pop
+    mb = np.nonzero(w.labels == 0)[0]
+    K.load_ephem(w.ephem.to_bytes())
+    for cap, want in ((40, kete.BODY_STEP_CAP), (400, 0)):
+        _form(K, form)
+        if form == "aside":   # (most of the attempts in the lanes, the rest in the warps)
+            K.set_propagation(0, kete.PROP_WORK_STEALING, 128, 8, 25)
+        st, ep = _dev(w.states[:, mb]), _dev(np.full(len(mb), W.T0 - 60.0))
+        status = K.propagate(st, ep, W.T0 + 800.0, fm=kete.force_model(max_steps=cap))
+        if form == "aside":
+            assert K.get_stats()["deferred"] > 0
+        assert (status.cpu().numpy() == want).all(), np.unique(status.cpu().numpy())
