@@ -580,9 +580,10 @@ static int make_grid(kete_ctx *ctx, const std::vector<double> &pts, double unit,
 // t_from: the first body's epoch, or where an earlier call left the chain
 // (NaN: not known).  use_grid: follow a step grid from t_from (from the first
 // stop where t_from is not known or lies past it) in units of about a day;
-// leg_days > 0: the grid's unit, its steps of one unit only.  Marks (kMarkRow)
-// between stops far apart cut the span into launches of at most kGridUnits
-// units.  Grid and marks lie on the table: an epoch off it fails its own body.
+// Marks (kMarkRow) between stops far apart cut the span into launches of at
+// most kGridUnits units.  Grid and marks lie on the table: an epoch off it fails
+// its own body.  leg_days > 0 (one stop, t_from known): stops that are not
+// written every leg_days from t_from on, which are the grid's points.
 static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const double *stops,
                      int n_stops, double t_from, double *out, int64_t stride, bool keep_on_fail,
                      bool use_grid, double leg_days = 0.0, bool out_aos = false)
@@ -624,13 +625,13 @@ static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const doub
         double prev = start;
         for (int k = 0; k < n_stops; k++) {
             const double from = leg_days > 0.0 ? prev : on_table(prev);
-            const double gap = (leg_days > 0.0 ? stops[k] : on_table(stops[k])) - from, most = unit * kGridUnits;
+            const double gap = (leg_days > 0.0 ? stops[k] : on_table(stops[k])) - from;
+            const double most = leg_days > 0.0 ? leg_days : unit * kGridUnits;
             const int64_t parts = (gap > 0.0) == forward ? (int64_t)std::ceil(std::fabs(gap) / most) : 0;
             for (int64_t p = 1; p < parts; p++) {
-                // on the leg grid, where there is one
-                const double step = leg_days > 0.0 ? (gap > 0 ? most : -most) : gap / (double)parts;
+                const double step = leg_days > 0.0 ? (forward ? most : -most) : gap / (double)parts;
                 m2.push_back(from + step * (double)p);
-                r2.push_back(kMarkRow);
+                r2.push_back(leg_days > 0.0 ? -1 : kMarkRow);
             }
             m2.push_back(stops[k]);
             r2.push_back(k);
@@ -656,15 +657,19 @@ static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const doub
                                 keep_on_fail, nullptr, out_aos);
     for (int k0 = 0; k0 < n_marks;) {
         int k1 = k0 + 1;   // the marks of this launch
-        while (k1 < n_marks && std::fabs(mark[k1] - start) <= unit * kGridUnits * (1.0 + 1e-12)) k1++;
+        while (k1 < n_marks && (leg_days > 0.0 ? k1 - k0 < kGridUnits
+                                               : std::fabs(mark[k1] - start) <= unit * kGridUnits * (1.0 + 1e-12)))
+            k1++;
         const double end = mark[k1 - 1], span = std::fabs(end - start);
         GridDev Q;
         const bool grid = end != start;
         if (grid) {
-            const int J = (int)std::max(1.0, std::min((double)kGridUnits, std::ceil(span / unit - 1e-9)));
+            const int J = leg_days > 0.0 ? k1 - k0
+                                         : (int)std::max(1.0, std::min((double)kGridUnits, std::ceil(span / unit - 1e-9)));
             const double u = leg_days > 0.0 ? leg_days : span / J;
             std::vector<double> pts((size_t)J + 1);
-            for (int j = 0; j <= J; j++) pts[j] = start + (end > start ? u : -u) * j;
+            for (int j = 0; j <= J; j++)
+                pts[j] = leg_days > 0.0 && j > 0 ? mark[k0 + j - 1] : start + (end > start ? u : -u) * j;
             pts[J] = end;
             const int r = make_grid(ctx, pts, u, leg_days > 0.0, Q);
             if (r != KETE_OK) return r;

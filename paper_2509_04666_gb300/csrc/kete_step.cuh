@@ -582,7 +582,8 @@ __device__ __forceinline__ int step_begin_grid(const EphemDev &E, const ForceDev
     // caller answers with plain steps)
     jn = on && j < Q.J ? j + 1 : j;
     if (fabs(dt) * Q.inv_unit >= 1.0) return step_aim(t, dt, __ldg(Q.g + jn), S, A);
-    const int st2 = step_aim(t, dt, __ldg(Q.g + Q.J), S, A);
+    // (a grid of single-unit legs: no step passes one)
+    const int st2 = step_aim(t, dt, __ldg(Q.g + (Q.n_len == 1 ? jn : Q.J)), S, A);
     while (jn < Q.J && (Q.dir > 0 ? __ldg(Q.g + jn) < A.t_new : __ldg(Q.g + jn) > A.t_new)) jn++;
     return st2;
 }
