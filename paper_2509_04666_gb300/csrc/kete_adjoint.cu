@@ -812,8 +812,10 @@ k_adj_observe(EphemDev E, AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
         auto newton = [&]() {
             const double d0 = pos[0] - ob.obs[0], d1 = pos[1] - ob.obs[1], d2 = pos[2] - ob.obs[2];
             const double range = sqrt(d0 * d0 + d1 * d1 + d2 * d2);
-            const double rate = (d0 * (vh[0] + svel[0]) + d1 * (vh[1] + svel[1]) +
-                                 d2 * (vh[2] + svel[2])) / range;
+            // (an observer on the body: no light time)
+            const double rate = range > 0.0 ? (d0 * (vh[0] + svel[0]) + d1 * (vh[1] + svel[1]) +
+                                               d2 * (vh[2] + svel[2])) / range
+                                            : 0.0;
             tau = (range + rate * tau) / (kC + rate);
         };
         ok = at(dt_obs) && ok;
