@@ -673,6 +673,7 @@ static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const doub
             pts[J] = end;
             const int r = make_grid(ctx, pts, u, leg_days > 0.0, Q);
             if (r != KETE_OK) return r;
+            Q.chain = n_stops > 1 || leg_days > 0.0;
         }
         const int r = propagate_launch(ctx, F, cs, start, end, d_stops + k0, d_row + k0, k1 - k0, out, stride,
                                        keep_on_fail, grid ? &Q : nullptr, out_aos);

@@ -75,6 +75,7 @@ struct GridDev {
     const uint8_t *ok;     // [step]
     double inv_unit;       // 1 / days per grid unit
     int J, n_len, nb, dir; // dir: +1 forward in time, -1 backward
+    int chain;             // the call has more than one stop
     int len[kGridLens];    // step lengths in grid units, ascending from 1
 };
 // stop_row of a mark: no stop of the caller's but where a launch ends.  Bodies

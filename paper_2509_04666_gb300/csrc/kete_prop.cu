@@ -541,14 +541,14 @@ static void launch_k(int64_t grid, int block, cudaStream_t st, const EphemDev &E
                      int n_stops, double *out, int64_t stride, int aos, int kof, DevCounters *ctr,
                      GridDev Q, int ug, unsigned long long *next, int refill, PropQueue q)
 {
-    // mixed precision on a grid: the node velocity in FP32 (V32)
+    // mixed precision along a chain of stops: the node velocity in FP32 (V32)
     if (F.nongrav) {
         k_propagate<MODE, true><<<(unsigned)grid, block, 0, st>>>(
             E, F, cs, stops, row, n_stops, out, stride, aos, kof, ctr, Q, ug, next, refill, q, FitRecord{});
         return;
     }
     if constexpr (MODE == KETE_MIXED) {
-        if (ug) {
+        if (ug && Q.chain) {
             k_propagate<MODE, false, true><<<(unsigned)grid, block, 0, st>>>(
                 E, F, cs, stops, row, n_stops, out, stride, aos, kof, ctr, Q, ug, next, refill, q, FitRecord{});
             return;
