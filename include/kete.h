@@ -380,7 +380,8 @@ int kete_set_propagation(kete_ctx *ctx, int precision, int kind, int block, int 
 /* Autotuner: time every launch variant (static 128, work stealing 64 and 128,
  * each in index and in cost order; work stealing 128 in cost order with long
  * bodies set aside after 64 or 24 attempts per stop) on an evenly spread sample of min(max_sample, n) of the n
- * bodies (device states [6][n] / epochs [n], not modified), run on persistent
+ * bodies (device states [6][n] / epochs [n], not modified), run in the form (lanes
+ * or warps) that a call of all n takes, on persistent
  * grids scaled down by sample / n so that each lane works through as many
  * bodies as in the whole run, propagated along
  * the chain of stops (host, ascending) with force model fm, keep the fastest

@@ -518,8 +518,8 @@ static int propagate_launch(kete_ctx *ctx, const ForceDev &F, ChainState cs, dou
     if (!(grid && grid->n_len == 1 && grid->J > 1) && warp_model(ctx->E, F, defer.model)) {
         GET(S_DEFER_LIST, cs.n, defer.list);
         GET(S_DEFER_CNT, 1, defer.count);
-        defer.budget0 = var.budget > 0 ? 0 : attempts_budget(ctx, cs.n, t_end - t_start,
-                                                                 F.precision == KETE_MIXED);
+        defer.budget0 = var.budget > 0 ? 0 : attempts_budget(ctx, var.population ? var.population : cs.n,
+                                                             t_end - t_start, F.precision == KETE_MIXED);
         dp = &defer;
     }
     int32_t *order = nullptr;
@@ -600,7 +600,7 @@ static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const doub
     ctx->stats.prop_budget = var.budget;
     ctx->stats.prop_order = var.order;
     WarpModel model;
-    const bool few = takes_warps(cs.n, stops[n_stops - 1] - t_from, F.precision == KETE_MIXED) &&
+    const bool few = takes_warps(var.population ? var.population : cs.n, stops[n_stops - 1] - t_from, F.precision == KETE_MIXED) &&
                      var.budget == 0 && leg_days == 0.0 && F.max_iter >= 8 &&
                      warp_model(ctx->E, F, model);
     if (few) use_grid = false;
@@ -1325,8 +1325,10 @@ extern "C" int kete_autotune(kete_ctx *ctx, const double *states, const double *
     if (r != KETE_OK) return r;
     F.nongrav = nullptr;   // the sample is gathered: body indices differ from the caller's
     CUDA_TRY(cudaSetDevice(ctx->device));
+    stats_begin(ctx);
     cudaStream_t st = ctx->stream;
-    // The sample (spread evenly over the bodies) runs on persistent grids scaled
+    // The sample (spread evenly over the bodies) runs in the form the whole would
+    // take and on persistent grids scaled
     // down by m / n, so that each lane works through as many bodies as in the
     // whole run: on the full grid a sample would leave a lane a few bodies and
     // be dominated by its longest-lived ones, which favours the split variants.
@@ -1339,7 +1341,7 @@ extern "C" int kete_autotune(kete_ctx *ctx, const double *states, const double *
     if ((r = first_epoch(ctx, epochs, e_first)) != KETE_OK) return r;
     CUDA_TRY(launch_gather_bodies(states, epochs, n, m, sst, sep, st));
     // schedules x cost order, then the split variants (with cost order)
-    PropVariant cands[9];
+    PropVariant cands[8];
     const int kinds[3][2] = {{PROP_STATIC, 128}, {PROP_WORK_STEALING, 64}, {PROP_WORK_STEALING, 128}};
     int n_cands = 0;
     for (int o = 0; o < 2; o++)
@@ -1347,18 +1349,23 @@ extern "C" int kete_autotune(kete_ctx *ctx, const double *states, const double *
             cands[n_cands] = PropVariant{kinds[q][0], kinds[q][1]};
             cands[n_cands++].order = o;
         }
-    const int splits[3][2] = {{8, 64}, {4, 64}, {8, 24}};
-    for (int q = 0; q < 3; q++) {
+    for (int budget : {64, 24}) {
         cands[n_cands] = PropVariant{PROP_WORK_STEALING, 128};
-        cands[n_cands].split = splits[q][0];
-        cands[n_cands].budget = splits[q][1];
+        cands[n_cands].split = 8;
+        cands[n_cands].budget = budget;
         cands[n_cands++].order = 1;
     }
+    // (the values of split act alike)
+    const auto alike = [](const PropVariant &a, const PropVariant &b) {
+        return a.kind == b.kind && a.block == b.block && (a.split > 0) == (b.split > 0) &&
+               a.budget == b.budget && a.order == b.order;
+    };
     const int slot = F.precision == KETE_MIXED ? 1 : 0;
     const PropVariant saved = ctx->var[slot];
     float best_ms = 1e30f, saved_ms = -1.0f;
     PropVariant best = saved;
-    cudaEvent_t e0 = event_at(ctx, 0), e1 = event_at(ctx, 1);
+    event_at(ctx, 3);
+    cudaEvent_t e0 = event_at(ctx, 2), e1 = event_at(ctx, 3);
     // time variant v on cnt bodies (states st, epochs ep; output rows out),
     // the best of reps runs after one that warms up
     auto time_variant = [&](const PropVariant &v, const double *st_, const double *ep_,
@@ -1369,7 +1376,6 @@ extern "C" int kete_autotune(kete_ctx *ctx, const double *states, const double *
             ChainState cs;
             int r2 = run_chain(ctx, F, st_, ep_, cnt, cs);
             if (r2 != KETE_OK) return r2;
-            CUDA_TRY(cudaMemsetAsync(ctx->d_ctr, 0, sizeof(DevCounters), st));
             CUDA_TRY(cudaEventRecord(e0, st));
             r2 = propagate(ctx, F, cs, stops, (int)n_stops, e_first, out_, cnt, false, true);
             if (r2 != KETE_OK) return r2;
@@ -1381,7 +1387,10 @@ extern "C" int kete_autotune(kete_ctx *ctx, const double *states, const double *
         }
         return KETE_OK;
     };
-    for (int c = 0; c < n_cands; c++) cands[c].grid_scale = scale;
+    for (int c = 0; c < n_cands; c++) {
+        cands[c].grid_scale = scale;
+        cands[c].population = n;
+    }
     for (int c = 0; c < n_cands; c++) {
         float ms;
         r = time_variant(cands[c], sst, sep, m, out, 2, ms);
@@ -1390,10 +1399,7 @@ extern "C" int kete_autotune(kete_ctx *ctx, const double *states, const double *
             best_ms = ms;
             best = cands[c];
         }
-        if (cands[c].kind == saved.kind && cands[c].block == saved.block &&
-            cands[c].split == saved.split && cands[c].budget == saved.budget &&
-            cands[c].order == saved.order)
-            saved_ms = ms;
+        if (alike(cands[c], saved)) saved_ms = ms;
     }
     // a sample ranks variants that differ by a few per cent unreliably (its
     // scaled-down grid holds fewer warps per SM than the real launch): the
@@ -1401,10 +1407,7 @@ extern "C" int kete_autotune(kete_ctx *ctx, const double *states, const double *
     // pick that does is checked against it on all the bodies when their
     // output rows fit in 2 GB
     if (saved_ms > 0.0f && best_ms > 0.95f * saved_ms) best = saved;
-    const bool same = best.kind == saved.kind && best.block == saved.block &&
-                      best.split == saved.split && best.budget == saved.budget &&
-                      best.order == saved.order;
-    if (!same && m < n && saved_ms > 0.0f && (double)n_stops * 48.0 * (double)n <= 2e9) {
+    if (!alike(best, saved) && m < n && saved_ms > 0.0f && (double)n_stops * 48.0 * (double)n <= 2e9) {
         double *full_out;
         GET(S_TUNE_OUT, (size_t)n_stops * 6 * n, full_out);
         PropVariant pick = best, cur = saved;
@@ -1419,7 +1422,10 @@ extern "C" int kete_autotune(kete_ctx *ctx, const double *states, const double *
         if (!(ms_pick < 0.98f * ms_cur)) best = saved;
     }
     best.grid_scale = 1.0;
-    ctx->var[F.precision == KETE_MIXED ? 1 : 0] = best;
+    best.population = 0;
+    ctx->var[slot] = best;
+    if ((r = stats_end(ctx)) != KETE_OK) return r;
+    stats_collect(ctx);   // the counters of all its runs
     if (kind) *kind = best.kind;
     if (block) *block = best.block;
     if (split_lanes) *split_lanes = best.split;

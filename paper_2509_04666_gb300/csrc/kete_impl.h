@@ -136,11 +136,13 @@ enum PropKind { PROP_STATIC = 0, PROP_WORK_STEALING = 1 };
 struct PropVariant {
     int kind;         // PropKind
     int block;        // threads per block (<= 128)
-    int split = 0;    // lanes per body for long bodies (4, 8, 16; 0 or 1: none)
+    int split = 0;    // > 1: the explicit budget below (the values 4, 8, 16 act alike)
     int budget = 0;   // step attempts per stop after which a body is set aside
     int order = 0;    // take bodies most expensive first (kete_order.cu)
     double grid_scale = 1.0;   // persistent grids scaled by this (<= 1: a sample of the
                                // bodies run with as many bodies per lane as the whole)
+    int64_t population = 0;    // bodies of the whole, which the form (lanes or warps) and the
+                               // set-aside budget follow (0: those of the call)
 };
 // stop_row (device, may be null): output row of each stop, -1: not written
 // (null: stop k is row k).  grid (may be null): the step grid to follow.
