@@ -10,6 +10,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -61,6 +62,7 @@ struct kete_ctx {
     int n_sm = 152;
     int pending_prop_pairs = 0;
     int64_t extra_launches = 0;     // ordering and second-phase launches of this call
+    std::vector<std::shared_ptr<const void>> uploads;   // host arrays that copies in flight read
     // phase timers: pairs of events per phase (prep, candidates, exact, order)
     std::vector<cudaEvent_t> phase_ev[4];
     int phase_n[4] = {0, 0, 0, 0};
@@ -147,6 +149,19 @@ static int get(kete_ctx *ctx, int s, size_t count, T **out)
         if (_r != KETE_OK) return _r;                      \
     } while (0)
 
+// Copy a host array to the device.  A copy from pageable memory may read it as
+// late as the stream gets to it (where the GPU reads host memory through the
+// host's page tables nothing is staged), so the context keeps it until it has
+// synchronised the stream.
+template <typename T>
+static cudaError_t upload(kete_ctx *ctx, T *dst, std::shared_ptr<const std::vector<T>> src)
+{
+    const cudaError_t e = cudaMemcpyAsync(dst, src->data(), src->size() * sizeof(T),
+                                          cudaMemcpyHostToDevice, ctx->stream);
+    ctx->uploads.push_back(std::move(src));
+    return e;
+}
+
 static cudaEvent_t event_at(kete_ctx *ctx, size_t i)
 {
     while (ctx->ev.size() <= i) {
@@ -159,6 +174,10 @@ static cudaEvent_t event_at(kete_ctx *ctx, size_t i)
 
 static void stats_begin(kete_ctx *ctx)
 {
+    if (!ctx->uploads.empty()) {   // left by a call that failed
+        cudaStreamSynchronize(ctx->stream);
+        ctx->uploads.clear();
+    }
     std::memset(&ctx->stats, 0, sizeof(ctx->stats));
     ctx->pending_prop_pairs = 0;
     ctx->extra_launches = 0;
@@ -185,6 +204,7 @@ static int stats_end(kete_ctx *ctx)
 static void stats_collect(kete_ctx *ctx)
 {
     cudaStreamSynchronize(ctx->stream);
+    ctx->uploads.clear();
     float ms = 0.0f;
     cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]);
     ctx->stats.total_ms = ms;
@@ -465,8 +485,7 @@ static int cost_order(kete_ctx *ctx, const double *states, int64_t stride, const
     GET(S_ORDER_OFF, nh + 1, s.off);
     GET(S_ORDER_SCAN, scan_tmp_elems((int64_t)nh), s.scan_tmp);
     GET(S_ORDER_N, 1, *order_n);
-    const unsigned long long nn = (unsigned long long)n;
-    CUDA_TRY(cudaMemcpyAsync(*order_n, &nn, sizeof(nn), cudaMemcpyHostToDevice, ctx->stream));
+    CUDA_TRY(upload(ctx, *order_n, std::make_shared<const std::vector<unsigned long long>>(1, n)));
     CUDA_TRY(order_by_cost(ctx->E, states, stride, epochs, n, t_end, t_end_i, ng, s, *order,
                            ctx->stream));
     ctx->extra_launches += order_launches(n, ng);
@@ -545,9 +564,11 @@ constexpr int kGridUnits = 512;   // units of one grid: 512 x 25 steps x 9 bodie
 constexpr double kGridMaxLaunches = 4096.0;   // grids of one call (5,700 years); longer spans take plain steps
 // The grid of one launch: points pts[0..J] (host, monotonic).  single: steps
 // of one unit only.
-static int make_grid(kete_ctx *ctx, const std::vector<double> &pts, double unit, bool single,
+static int make_grid(kete_ctx *ctx, std::vector<double> &&points, double unit, bool single,
                      GridDev &Q)
 {
+    const auto shared = std::make_shared<const std::vector<double>>(std::move(points));
+    const std::vector<double> &pts = *shared;
     const int J = (int)pts.size() - 1;
     Q = GridDev{};
     Q.J = J;
@@ -565,8 +586,7 @@ static int make_grid(kete_ctx *ctx, const std::vector<double> &pts, double unit,
     GET(S_GRID_R64, elems, r64);
     GET(S_GRID_R32, elems, r32);
     GET(S_GRID_OK, steps, ok);
-    CUDA_TRY(cudaMemcpyAsync(g, pts.data(), (J + 1) * sizeof(double), cudaMemcpyHostToDevice,
-                             ctx->stream));
+    CUDA_TRY(upload(ctx, g, shared));
     Q.g = g;
     Q.row64 = r64;
     Q.row32 = r32;
@@ -588,7 +608,7 @@ static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const doub
                      int n_stops, double t_from, double *out, int64_t stride, bool keep_on_fail,
                      bool use_grid, double leg_days = 0.0, bool out_aos = false)
 {
-    std::vector<double> mark(stops, stops + n_stops);
+    std::vector<double> at(stops, stops + n_stops);
     std::vector<int32_t> row((size_t)n_stops);
     for (int k = 0; k < n_stops; k++) row[k] = k;
     double *d_stops;
@@ -637,16 +657,16 @@ static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const doub
             r2.push_back(k);
             prev = stops[k];
         }
-        mark.swap(m2);
+        at.swap(m2);
         row.swap(r2);
     }
+    const auto marks = std::make_shared<const std::vector<double>>(std::move(at));
+    const std::vector<double> &mark = *marks;
     const int n_marks = (int)mark.size();
     GET(S_STOPS, n_marks, d_stops);
     GET(S_STOPROW, n_marks, d_row);
-    CUDA_TRY(cudaMemcpyAsync(d_stops, mark.data(), n_marks * sizeof(double), cudaMemcpyHostToDevice,
-                             ctx->stream));
-    CUDA_TRY(cudaMemcpyAsync(d_row, row.data(), n_marks * sizeof(int32_t), cudaMemcpyHostToDevice,
-                             ctx->stream));
+    CUDA_TRY(upload(ctx, d_stops, marks));
+    CUDA_TRY(upload(ctx, d_row, std::make_shared<const std::vector<int32_t>>(std::move(row))));
     if (few) {
         CUDA_TRY(launch_propagate_warp(ctx->E, F, model, cs, d_stops, d_row, n_marks, out, stride,
                                        keep_on_fail, ctx->d_ctr, ctx->stream, PropQueue{}, out_aos));
@@ -671,7 +691,7 @@ static int propagate(kete_ctx *ctx, const ForceDev &F, ChainState cs, const doub
             for (int j = 0; j <= J; j++)
                 pts[j] = leg_days > 0.0 && j > 0 ? mark[k0 + j - 1] : start + (end > start ? u : -u) * j;
             pts[J] = end;
-            const int r = make_grid(ctx, pts, u, leg_days > 0.0, Q);
+            const int r = make_grid(ctx, std::move(pts), u, leg_days > 0.0, Q);
             if (r != KETE_OK) return r;
             Q.chain = n_stops > 1 || leg_days > 0.0;
         }
@@ -1555,7 +1575,7 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
                     std::vector<double> pts((size_t)J + 1);
                     for (int j = 0; j <= J; j++) pts[j] = lo + span / J * j;
                     pts[J] = hi;
-                    if ((r = make_grid(ctx, pts, span / J, false, Q)) != KETE_OK) return r;
+                    if ((r = make_grid(ctx, std::move(pts), span / J, false, Q)) != KETE_OK) return r;
                 }
             }
             if (order_on && (!warps || lanes)) {   // most expensive bodies first (schedule only)

@@ -74,8 +74,8 @@ static inline void fill_radau_tables(RadauTables &t)
 // fill this translation unit's copy of g_rt
 static inline cudaError_t upload_step_tables(cudaStream_t st)
 {
-    RadauTables t;
-    fill_radau_tables(t);
+    // (static: the copy may read it after the return)
+    static const RadauTables t = [] { RadauTables r; fill_radau_tables(r); return r; }();
     return cudaMemcpyToSymbolAsync(g_rt, &t, sizeof(t), 0, cudaMemcpyHostToDevice, st);
 }
 

@@ -40,7 +40,7 @@ struct WarpTables {
 };
 static __constant__ WarpTables g_wt;
 
-cudaError_t upload_warp_tables(cudaStream_t st)
+static WarpTables warp_tables()
 {
     RadauTables t;
     fill_radau_tables(t);
@@ -58,6 +58,12 @@ cudaError_t upload_warp_tables(cudaStream_t st)
             (n < 8 ? w.wv[n] : w.wve)[k] = (double)av;
         }
     }
+    return w;
+}
+
+cudaError_t upload_warp_tables(cudaStream_t st)
+{
+    static const WarpTables w = warp_tables();   // (the copy may read it after the return)
     cudaError_t e = upload_step_tables(st);
     if (e != cudaSuccess) return e;
     return cudaMemcpyToSymbolAsync(g_wt, &w, sizeof(w), 0, cudaMemcpyHostToDevice, st);
