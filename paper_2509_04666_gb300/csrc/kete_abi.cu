@@ -1591,7 +1591,9 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
                 PropDefer defer{};
                 GET(S_DEFER_LIST, nc, defer.list);
                 GET(S_DEFER_CNT, 1, defer.count);
-                defer.budget0 = attempts_budget(ctx, nc, span, false);
+                // (lengths rounded down to the grid's can double a body's steps: one
+                // near the record limit takes its own in a warp)
+                defer.budget0 = std::min(attempts_budget(ctx, nc, span, false), KETE_ADJ_MAX_STEPS / 2);
                 CUDA_TRY(launch_fit_lanes(ctx->E, F, B, P, i0, nc, Q, next, order, order_n, defer,
                                           ctx->stream));
                 CUDA_TRY(launch_fit_jacobian(ctx->E, F, B, nc, ctx->stream));

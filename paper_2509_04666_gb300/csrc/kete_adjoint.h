@@ -59,6 +59,21 @@ struct AdjBuffers {
 // lanes of the forward pass's grid for chunks of nc bodies
 int64_t adjoint_forward_lanes(int64_t nc, bool full);
 
+// checkpoints of the grid before t
+__device__ __forceinline__ double ckpts_before(double ckpt, double epoch0, double t)
+{
+    return ckpt > 0.0 && t > epoch0 ? ceil((t - epoch0) / ckpt) - 1.0 : 0.0;
+}
+
+// The record limit counts steps that end at every stop, midpoint and checkpoint
+// (k_adj_forward's): a step that passes stops is one for each of them, the others
+// one.  (Stops and steps added up would refuse arcs whose every step is a leg: 4
+// years of 8-day legs, 183 steps there, came to 281.)
+__device__ __forceinline__ int steps_with_stops(double ckpts, int midpoints)
+{
+    return max(1, (int)fmin(ckpts, 1e6) + midpoints);
+}
+
 // observations in use: those before the first non-finite epoch
 __device__ __forceinline__ int obs_count(const kete_obs *o, int m)
 {

@@ -111,15 +111,13 @@ __device__ __forceinline__ void fit_stop(const FitRecord &R, int k, int64_t i, i
     R.B.bfrac[at] = frac;
 }
 
-// the body's last record (its final state) and status; the checkpoint grid's
-// stops count toward the record limit
+// the body's last record (its final state) and status; used: its steps counted
+// toward the record limit (steps_with_stops)
 __device__ __forceinline__ void fit_done(const EphemDev &E, const FitRecord &R, int64_t i, int status, bool capped,
-                                         int count, int n_stops, double epoch0, double t,
-                                         const double x[3], double *rec)
+                                         int count, int used, double t, const double x[3],
+                                         double *rec)
 {
-    if (R.P.ckpt > 0.0 && t > epoch0 &&
-        count + n_stops + ceil((t - epoch0) / R.P.ckpt) - 1.0 > (double)(R.B.cap - 1))
-        capped = true;
+    if (R.P.ckpt > 0.0 && used > R.B.cap - 1) capped = true;
     Seg g;
     if (status == KETE_BODY_OK && capped) status = KETE_BODY_ADJ_CAP;
     else if (status == KETE_BODY_OK && !ephem_seg(E, t, 0.0, g)) status = KETE_BODY_OUT_OF_SPAN;
@@ -151,7 +149,7 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
     const double *stops = stops_in;   // its stops
     int n_stops = n_stops_in;
     double *rec = nullptr, epoch0 = 0.0;   // REC: its records
-    int count = 0;
+    int count = 0, used = 0;
     bool capped = false;
     int k = 0;                // next stop of the body
     double x[3], v[3], t = 0.0, dt = 0.0;
@@ -181,6 +179,7 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                     bool accepted;
                     status = step_control<MODE>(F, A, x, v, dt, S, cnt, x1, v1, accepted);
                     if (accepted) {
+                        const int k_from = k;
                         if (!plain) {
                             // stops inside the step, from its polynomial
                             while (k < n_stops && (Q.dir > 0 ? stops[k] < A.t_new : stops[k] > A.t_new)) {
@@ -200,6 +199,9 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                                 dt = proposed;
                         }
                         if (REC) {   // the step's polynomial (k_fit_jacobian turns it into da/dx)
+                            const double ck = ckpts_before(R.P.ckpt, epoch0, A.t_new) -
+                                              ckpts_before(R.P.ckpt, epoch0, t);
+                            used += steps_with_stops(ck, k - k_from + (k < n_stops && stops[k] == A.t_new));
                             if (count < R.B.cap - 1) {
                                 double *r = rec + (size_t)count * kAdjRec;
                                 r[0] = t;
@@ -272,7 +274,7 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                                 n_stops = R.B.nbat[i];
                                 capped = R.B.n_rec[i] != 0;
                                 rec = R.B.rec + (size_t)i * R.B.cap * kAdjRec;
-                                count = 0;
+                                count = used = 0;
                             } else {
 #pragma unroll
                                 for (int c = 0; c < 3; c++) {
@@ -340,7 +342,7 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                             atomicAdd(&ctr->deferred, 1ull);
                             R.B.n_rec[i] = 0;
                         } else {
-                            fit_done(E, R, i, status, capped, count, n_stops, epoch0, t, x, rec);
+                            fit_done(E, R, i, status, capped, count, used, t, x, rec);
                         }
                         phase = TAKE;
                     } else if (k >= n_stops || aside) {

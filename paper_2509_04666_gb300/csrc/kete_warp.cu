@@ -293,7 +293,7 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
         const int64_t i = q.list ? (int64_t)q.list[item] : (int64_t)item;
         // own coordinate of the step-start state
         double x0, v0, t, dt = 0.0;
-        int status = KETE_BODY_OK, k = 0, count = 0;
+        int status = KETE_BODY_OK, k = 0, count = 0, used = 0;
         double *rec = nullptr;
         bool capped = false;
         if (REC) {
@@ -657,6 +657,7 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
                     capped = true;
                 }
             }
+            const int k_from = k;
             // stops inside the step, eight at a time (node group q takes stop k + q)
             if (fwd && !careful && stops[k] < t_new) {
                 double b[7];
@@ -697,6 +698,11 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
                 }
                 attempts = 0;
             }
+            if (REC) {
+                const double ck = ckpts_before(R.P.ckpt, epoch0, t_new) -
+                                  ckpts_before(R.P.ckpt, epoch0, t);
+                used += steps_with_stops(ck, k - k_from + (k < n_stops && stops[k] == t_new));
+            }
             x0 = x1;
             v0 = v1;
             t = t_new;
@@ -705,9 +711,7 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
             if (REC && count < R.B.cap - 1) count++;
         }
         if (REC) {
-            if (R.P.ckpt > 0.0 && t > epoch0 &&
-                count + n_stops + ceil((t - epoch0) / R.P.ckpt) - 1.0 > (double)(R.B.cap - 1))
-                capped = true;
+            if (R.P.ckpt > 0.0 && used > R.B.cap - 1) capped = true;
             if (status == KETE_BODY_OK && !capped) {   // da/dx at the final state closes the last step
                 const bool inside = lane_planets(E, W, t, 0.0, M);
                 const double zero[3] = {0.0, 0.0, 0.0};
