@@ -202,6 +202,7 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                             const double ck = ckpts_before(R.P.ckpt, epoch0, A.t_new) -
                                               ckpts_before(R.P.ckpt, epoch0, t);
                             used += steps_with_stops(ck, k - k_from + (k < n_stops && stops[k] == A.t_new));
+                            if (ck > 0.0) attempts = 0;   // max_steps counts the attempts of a leg
                             if (count < R.B.cap - 1) {
                                 double *r = rec + (size_t)count * kAdjRec;
                                 r[0] = t;

@@ -702,6 +702,7 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
                 const double ck = ckpts_before(R.P.ckpt, epoch0, t_new) -
                                   ckpts_before(R.P.ckpt, epoch0, t);
                 used += steps_with_stops(ck, k - k_from + (k < n_stops && stops[k] == t_new));
+                if (ck > 0.0) attempts = 0;   // max_steps counts the attempts of a leg
             }
             x0 = x1;
             v0 = v1;

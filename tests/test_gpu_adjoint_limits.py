@@ -1,9 +1,10 @@
-"""The limits of an orbit fit over long arcs: what the steps
+"""The limits of an orbit fit over long arcs and with few attempts: what the steps
 that end at every midpoint and checkpoint (force models of seven corrector
 iterations take them) allow, the forms whose steps pass them allow too.  A
 main-belt body's own steps are 10 to 25 days long, so with checkpoints every 8 days
 each is one step: 4 years of them are 183 of the 255, 500 days of 2.2-day ones 228,
-and a step cut short by a midpoint costs a few more."""
+and a step cut short by a midpoint costs a few more; no leg needs more than its
+first step's few attempts."""
 import numpy as np
 import pytest
 
@@ -28,7 +29,8 @@ def K():
 
 @pytest.mark.parametrize("days,m,ckpt,cap,copies", [
     (1460.0, 1, 8.0, 100_000, 1), (1460.0, 5, 8.0, 100_000, 1), (500.0, 1, 2.2, 100_000, 1),
-    (500.0, 1, 2.2, 100_000, 1000)])
+    (500.0, 1, 2.2, 100_000, 1000),
+    (90.0, 1, 8.0, 5, 1), (90.0, 1, 8.0, 5, 1000)])
 def test_arcs_that_fit_the_stops_are_accepted(K, days, m, ckpt, cap, copies):
     from paper_2509_04666_gb300 import kete
     n = 18
