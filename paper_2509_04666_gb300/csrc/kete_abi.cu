@@ -32,7 +32,7 @@ enum Slot {
     S_GRID_R64, S_GRID_R32, S_STOPROW, S_XSUN, S_XOBSREL, S_NEXTBODY, S_TUNE_ST, S_TUNE_EP, S_TUNE_OUT,
     S_ADJ_REC, S_ADJ_NREC, S_ADJ_NBAT, S_ADJ_BIDX, S_ADJ_YREF, S_ADJ_GJUMP, S_ADJ_STATUS,
     S_KSTOP, S_TRIES, S_DEFER_LIST, S_DEFER_CNT, S_ORDER, S_ORDER_KEY, S_ORDER_HIST, S_ORDER_OFF,
-    S_ORDER_SCAN, S_ORDER_N, S_ADJ_TEND, S_LEG_OUT,
+    S_ORDER_SCAN, S_ORDER_N, S_ADJ_TEND,
     S_EXT_START, S_EXT_EX, S_EXT_TMP, S_EXT_FIRST, S_EXT_SUB, S_EXT_PARENT, S_EXT_CNT,
     S_EXT_OFF, S_EXT_CUR, S_EXT_GROUP, S_EXT_KEEP, S_EXT_KCNT, S_EXT_KOFF, S_ADJ_PHI, S_ADJ_RECX,
     S_PRE_KEEP, S_PRE_N, S_ADJ_RICH, S_ADJ_PLANETS, S_ADJ_BFRAC, S_ADJ_MID, S_ADJ_RANGE,

@@ -1390,7 +1390,7 @@ k_adj_backward_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 // with F_k = h^2 (Ax dx_k + Av dv_k) at the samples (node 0..7, step end):
 //   dx(s_n) = dx_0 + s_n h dv_0 + sum_k W2f[n][k] F_k,
 //   dv(s_n) = dv_0 + (1/h) sum_k W1f[n][k] F_k,
-// Gauss-Seidel sweeps as in k_adj_backward_full.
+// Gauss-Seidel sweeps as in k_adj_backward_full.  Its steps end at the batch midpoints.
 __global__ void __launch_bounds__(128)
 k_adj_stm_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 {
@@ -1406,13 +1406,12 @@ k_adj_stm_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
     const int32_t *bidx = B.bidx + (size_t)i * P.m;
     double *phi_out = B.phi + (size_t)i * P.m * 36;
     {
-        const double *bfrac = B.bfrac + (size_t)i * P.m;
         double dx[3] = {0, 0, 0}, dv[3] = {0, 0, 0};
         if (c0 < 3) dx[c0] = 1.0;
         else dv[c0 - 3] = 1.0;
         int kb = 0;
         for (int s = 0; s <= count - 1; s++) {
-            while (kb < nb && bidx[kb] == s && (bfrac[kb] == 0.0 || s == count - 1)) {
+            while (kb < nb && bidx[kb] == s) {
                 store_column(phi_out + (size_t)kb * 36, c0, dx, dv);
                 kb++;
             }
@@ -1468,12 +1467,6 @@ k_adj_stm_full(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
                                  F[n]);
                 }
                 if (colloc_done(delta, size, before)) break;
-            }
-// midpoints inside the step
-            for (; kb < nb && bidx[kb] == s; kb++) {
-                double xs[3], vs[3];
-                colloc_at(F, h, bfrac[kb], dx, dv, xs, vs);
-                store_column(phi_out + (size_t)kb * 36, c0, xs, vs);
             }
 #pragma unroll
             for (int c = 0; c < 3; c++) {
