@@ -1495,6 +1495,7 @@ static int adjoint_impl(kete_ctx *ctx, const double *states, const double *epoch
         P.m = m;
         P.span = std::min(opt.batch_span, 2.0 * opt.twobody_max);
         P.ckpt = ckpt_days;
+        P.inv_ckpt = ckpt_days > 0.0 ? 1.0 / ckpt_days : 0.0;
         P.cos_eps = std::cos(eps_obl);
         P.sin_eps = std::sin(eps_obl);
         P.loss = loss;

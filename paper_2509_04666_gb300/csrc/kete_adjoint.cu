@@ -3,22 +3,26 @@
 // Sec. 2: n-body propagation of App. A, two-body + light time, RA/Dec).
 //
 // Three kernels per chunk of bodies:
-//   forward pass    k_propagate_warp (kete_warp.cu), or k_adj_forward, one lane
-//                   per body at a time (work stealing), with non-gravitational
-//                   terms and for force models the warp form does not serve.
+//   forward pass    in one of three forms: k_propagate_warp (kete_warp.cu), one
+//                   warp per body; for many bodies whose chains share a step
+//                   grid the lanes of k_propagate (kete_prop.cu) between
+//                   k_fit_stops and k_fit_jacobian, long bodies set aside for
+//                   the warps; k_adj_forward, one lane per body at a time (work
+//                   stealing), with non-gravitational terms and for force
+//                   models the warp form does not serve.
 //                   The body's observations are batched
 //                   by the <= span rule (Sec. 2); the chain visits the batch
-//                   midpoints (k_adj_forward: and the checkpoint grid) in
-//                   ascending order with Gauss-Radau steps; k_propagate_warp
-//                   takes the midpoints inside a step from its polynomial.
+//                   midpoints in ascending order with Gauss-Radau steps.
+//                   k_adj_forward's end there and at the checkpoints; the other
+//                   two take the midpoints inside a step from its polynomial.
 //                   Every accepted step leaves a record in device memory: its
 //                   start and end epochs and the Newtonian da/dx at its 8
-//                   Gauss-Radau nodes, taken from the force evaluations the
-//                   step already makes.  The state at each batch midpoint is
+//                   Gauss-Radau nodes (k_fit_jacobian forms them from the
+//                   recorded polynomials).  The state at each batch midpoint is
 //                   kept for the sky projection.
 //   k_adj_observe   one thread per observation: prediction,
 //                   residual, loss term and dL/dy(t_ref) through RA/Dec, the
-//                   light-time fixed point (implicit derivative) and the
+//                   light time (Newton; implicit derivative) and the
 //                   universal-variable two-body map (forward-mode dual numbers
 //                   at the converged universal anomaly).
 //   k_adj_backward  one lane per body: (lambda_x, lambda_v) carried back over
@@ -744,9 +748,9 @@ __device__ __forceinline__ double wrap_pi(double a)
 }
 
 // Thread per observation slot, 128 / m whole bodies to a block of 128 threads:
-// FP64 issue bounds it (5 two-body solves an observation), and a warp per body
-// left 12 of 32 lanes idle at 20 observations (100,000 bodies: 17.0 ms, now
-// 11.5).  w: the body within the block, lane: its observation.
+// FP64 issue bounds it (3 two-body solves an observation), and a warp per body
+// left 12 of 32 lanes idle at 20 observations (100,000 bodies, 5 solves: 17.0 ms
+// and 11.5 this way).  w: the body within the block, lane: its observation.
 __global__ void __launch_bounds__(128)
 k_adj_observe(EphemDev E, AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 {
@@ -812,11 +816,10 @@ k_adj_observe(EphemDev E, AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
         auto newton = [&]() {
             const double d0 = pos[0] - ob.obs[0], d1 = pos[1] - ob.obs[1], d2 = pos[2] - ob.obs[2];
             const double range = sqrt(d0 * d0 + d1 * d1 + d2 * d2);
-            // (an observer on the body: no light time)
-            const double rate = range > 0.0 ? (d0 * (vh[0] + svel[0]) + d1 * (vh[1] + svel[1]) +
-                                               d2 * (vh[2] + svel[2])) / range
-                                            : 0.0;
+            const double rate = (d0 * (vh[0] + svel[0]) + d1 * (vh[1] + svel[1]) +
+                                 d2 * (vh[2] + svel[2])) / range;
             tau = (range + rate * tau) / (kC + rate);
+            if (range == 0.0) tau = 0.0;   // an observer on the body
         };
         ok = at(dt_obs) && ok;
         newton();
@@ -983,7 +986,7 @@ __device__ __forceinline__ bool colloc_done(double delta, double size, double &b
 // end (W2f is nearly lower triangular; contraction ~ h^2 |J|), at most 12.
 // FP64 issue bounds it: a sweep is 330 multiply-adds, a midpoint 220.  With the
 // forward pass stopping at no midpoint (6-7 steps instead of 25 over 90 days and
-// 20 midpoints), 100,000 bodies: loss and gradient 164 -> 68.6 ms.
+// 20 midpoints), 100,000 bodies: 8.4 ms.
 __global__ void __launch_bounds__(128)
 k_adj_backward(AdjBuffers B, AdjProblem P, int64_t i0, int64_t nc)
 {

@@ -23,7 +23,7 @@ struct AdjProblem {
     int64_t n;
     const kete_obs *obs;
     int32_t m;
-    double span, ckpt;
+    double span, ckpt, inv_ckpt;   // inv_ckpt: 1 / ckpt (0: no grid)
     double cos_eps, sin_eps;
     double *loss, *grad, *pred;
     double *jac;       // [n][m][2][6] d(RA, Dec)/d(x0, v0) per observation, or null
@@ -59,10 +59,10 @@ struct AdjBuffers {
 // lanes of the forward pass's grid for chunks of nc bodies
 int64_t adjoint_forward_lanes(int64_t nc, bool full);
 
-// checkpoints of the grid before t
-__device__ __forceinline__ double ckpts_before(double ckpt, double epoch0, double t)
+// checkpoints of the grid (one in 1 / inv_ckpt days, none for 0) before t
+__device__ __forceinline__ double ckpts_before(double inv_ckpt, double epoch0, double t)
 {
-    return ckpt > 0.0 && t > epoch0 ? ceil((t - epoch0) / ckpt) - 1.0 : 0.0;
+    return inv_ckpt > 0.0 && t > epoch0 ? ceil((t - epoch0) * inv_ckpt) - 1.0 : 0.0;
 }
 
 // The record limit counts steps that end at every stop, midpoint and checkpoint

@@ -199,8 +199,8 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                                 dt = proposed;
                         }
                         if (REC) {   // the step's polynomial (k_fit_jacobian turns it into da/dx)
-                            const double ck = ckpts_before(R.P.ckpt, epoch0, A.t_new) -
-                                              ckpts_before(R.P.ckpt, epoch0, t);
+                            const double ck = ckpts_before(R.P.inv_ckpt, epoch0, A.t_new) -
+                                              ckpts_before(R.P.inv_ckpt, epoch0, t);
                             used += steps_with_stops(ck, k - k_from + (k < n_stops && stops[k] == A.t_new));
                             if (ck > 0.0) attempts = 0;   // max_steps counts the attempts of a leg
                             if (count < R.B.cap - 1) {

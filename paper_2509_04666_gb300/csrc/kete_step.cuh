@@ -431,8 +431,8 @@ struct StepState {
 // They start a step's corrector: from the constant a0 the first sweep's nodes
 // are off by ~(n h)^3 of a, with these by what the planets change over the
 // step, for ~60 operations against a sweep's ~2,700 (main belt: 3.7 sweeps a
-// step without, 3.0 with them at a ten times tighter threshold).  Nothing is
-// extrapolated from the step before.
+// step without, 3.0 with them at a ten times tighter threshold).  Used where no
+// step of like length went before (START_NEXT) and in mixed precision.
 __device__ __forceinline__ void two_body_derivs(double mu, const double r[3], const double w[3],
                                                 double d1[3], double d2[3], double d3[3])
 {

@@ -4,8 +4,8 @@
 //
 // An FP64 warp instruction occupies its SM sub-partition's FP64 unit for 64
 // cycles whatever its active lanes, so a lane-per-body step is a serial chain
-// of about 29 force evaluations x 650 FP64 instructions: 0.8 ms, and the
-// slowest body of a call sets its time.  Here the 32 lanes of a warp share one
+// of 15-16 force evaluations x 250 FP64 instructions on the grid's rows (650
+// off it): 0.4 ms, and the slowest body of a call sets its time.  Here the 32 lanes of a warp share one
 // body's step: lane 4 n + r holds Gauss-Radau node n (0: the step start) and
 // every fourth mass from r on, and coordinate r of the corrector.
 //   - The planets at the 8 nodes are summed once per attempt and kept in
@@ -699,8 +699,8 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
                 attempts = 0;
             }
             if (REC) {
-                const double ck = ckpts_before(R.P.ckpt, epoch0, t_new) -
-                                  ckpts_before(R.P.ckpt, epoch0, t);
+                const double ck = ckpts_before(R.P.inv_ckpt, epoch0, t_new) -
+                                  ckpts_before(R.P.inv_ckpt, epoch0, t);
                 used += steps_with_stops(ck, k - k_from + (k < n_stops && stops[k] == t_new));
                 if (ck > 0.0) attempts = 0;   // max_steps counts the attempts of a leg
             }
