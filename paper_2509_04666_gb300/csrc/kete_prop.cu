@@ -227,7 +227,7 @@ k_propagate(EphemDev E, ForceDev F, ChainState cs, const double *__restrict__ st
                         }
                         t = A.t_new;
                         S.have_a0 = false;
-                        S.chained = true;
+                        S.chained = fabs(dt) <= kNextMost * fabs(A.h);
                     } else {
                         S.start = MODE == KETE_MIXED ? START_A0 : START_RETRY;
                     }

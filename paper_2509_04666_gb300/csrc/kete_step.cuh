@@ -148,13 +148,15 @@ struct Attempt {
 // (FP64 only: START_NEXT, START_RETRY)
 // START_NEXT only for a step of at most kNextMost times the last one: continued
 // q steps far, b6 grows q^7-fold, and after a short step (to a grid point, to a
-// segment boundary) its b6 is rounding.  The sweeps correct b by increments, so
-// what rounding leaves of an absurd start stays in the solution: 400 bodies
-// whose first step is 0.0015 days and whose second is 1 day ended 60 days on
-// 1e-6 AU off, 1e-15 within this bound.  Step control grows a step by at most
-// 1 / safety, 4 by default.
+// segment boundary) its b6 is rounding, 1e-13 |a|.  The sweeps correct b by
+// increments, so what rounding leaves of an absurd start stays in the solution:
+// 400 bodies whose first step is 0.0015 days and whose second is 1 day ended 60
+// days on 1e-6 AU off, 1e-15 within this bound.  At 16 the start is 3e-5 |a| off, no
+// more than the two-body one; step control grows a step by at most 1 / safety, 4
+// by default (a bound of 4, met by steps to grid points, cost 99,000 mixed bodies
+// over 400 days 82.8 ms, 16 costs 77.3).
 enum CorrectorStart { START_A0, START_DERIVS, START_NEXT, START_RETRY };
-constexpr double kNextMost = 4.0;
+constexpr double kNextMost = 16.0;
 
 // coefficients b of sum b_k s^(k+1) in s' of s = next + q s' (next 1 or 0), the
 // constant dropped: b'_k = q^(k+1) (b_k + next sum_{j>k} C(j+1, k+1) b_j)
@@ -416,7 +418,8 @@ struct StepState {
     double bound;           // epoch no step may pass: the next table segment boundary
                             // during an encounter, else infinite
     int start;              // what the next attempt's corrector starts from (CorrectorStart)
-    bool chained;           // the Attempt holds an accepted step that ended here
+    bool chained;           // the Attempt holds an accepted step that ended here, and the
+                            // next one is proposed within kNextMost times its length
     bool have_a0;           // a0 valid for (x, v, t): kept across a rejection
     const kete_nongrav *ng; // the body's non-gravitational terms (null: none)
     double ng_chi;          // the thermal lag's last two-body solution (0: none yet)
@@ -454,16 +457,16 @@ __device__ __forceinline__ void two_body_derivs(double mu, const double r[3], co
     }
 }
 
-// The acceleration at the start of a step attempt of (x, v, t) of at most |dt|
-// if it is not known yet (kept across a rejection), from node-0 rows when given,
+// The acceleration at the start of a step attempt of (x, v, t) if it is not
+// known yet (kept across a rejection), from node-0 rows when given,
 // what its corrector starts from (S.start; the derivatives in A.b), and the
 // epoch no step toward `dir` may pass: during an encounter no step straddles
 // a boundary of the planet polynomials (S.bound; infinite otherwise).
 template <int MODE, bool JAC>
 __device__ __forceinline__ int step_start(const EphemDev &E, const ForceDev &F, const double *r64,
                                           const float *r32, const double x[3], const double v[3],
-                                          double t, double dt, bool forward, StepState &S,
-                                          Attempt &A, Cnt &cnt, double *jrec)
+                                          double t, bool forward, StepState &S, Attempt &A,
+                                          Cnt &cnt, double *jrec)
 {
     if (S.have_a0) {
         S.start = JAC ? START_A0 : S.start;
@@ -485,7 +488,7 @@ __device__ __forceinline__ int step_start(const EphemDev &E, const ForceDev &F, 
         S.bound = b;
     }
     S.start = START_A0;
-    if (!JAC && MODE == KETE_FP64 && S.chained && fabs(dt) <= kNextMost * fabs(A.h)) {
+    if (!JAC && MODE == KETE_FP64 && S.chained) {
         S.start = START_NEXT;
     } else if (!JAC && (F.active_mask & 1u)) {
         S.start = START_DERIVS;
@@ -520,7 +523,7 @@ __device__ __forceinline__ int step_begin(const EphemDev &E, const ForceDev &F, 
                                           StepState &S, Attempt &A, Cnt &cnt,
                                           double *jrec = nullptr)
 {
-    const int st = step_start<MODE, JAC>(E, F, nullptr, nullptr, x, v, t, dt, target > t, S, A,
+    const int st = step_start<MODE, JAC>(E, F, nullptr, nullptr, x, v, t, target > t, S, A,
                                             cnt, jrec);
     return st != KETE_BODY_OK ? st : step_aim(t, dt, target, S, A);
 }
@@ -556,8 +559,8 @@ __device__ __forceinline__ int step_begin_grid(const EphemDev &E, const ForceDev
     const bool row0 = on && j < Q.J && __ldg(Q.ok + (size_t)j * Q.n_len);
     const size_t at0 = (size_t)j * Q.n_len * cell;
     const int st = step_start<MODE, false>(E, F, row0 ? Q.row64 + at0 : nullptr,
-                                              row0 ? Q.row32 + at0 : nullptr, x, v, t, dt, Q.dir > 0,
-                                              S, A, cnt, nullptr);
+                                              row0 ? Q.row32 + at0 : nullptr, x, v, t, Q.dir > 0, S, A,
+                                              cnt, nullptr);
     if (st != KETE_BODY_OK) return st;
     if (on) {
         const double units = fabs(dt) * Q.inv_unit * (1.0 + 1e-12);

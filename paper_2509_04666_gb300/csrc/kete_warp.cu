@@ -450,8 +450,8 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
                 const int s2 = own_terms(node == 0, xs, vs, own);
                 const double f = node_force(W, M, xs, vs, zero, -1, d0, r, own);
                 a0 = __shfl_sync(kFull, f, r);
-                start = chained && fabs(h) <= kNextMost * fabs(h_last) ? START_NEXT : START_DERIVS;
-                if (start == START_DERIVS) {   // two_body_derivs, from the Sun in lane 0
+                start = chained ? START_NEXT : START_DERIVS;
+                if (!chained) {   // two_body_derivs, from the Sun in lane 0
                     double hr[3], hw[3], e1[3], e2[3], e3[3];
 #pragma unroll
                     for (int c = 0; c < 3; c++) {
@@ -708,7 +708,7 @@ k_propagate_warp(EphemDev E, ForceDev F, WarpModel W, ChainState cs,
             v0 = v1;
             t = t_new;
             have_a0 = false;
-            chained = true;
+            chained = factor <= kNextMost;
             if (REC && count < R.B.cap - 1) count++;
         }
         if (REC) {
