@@ -112,7 +112,9 @@ typedef struct kete_force_model {
     double dt_init;              /* first step of each propagation chain, days (4) */
     int32_t max_iter;            /* corrector iteration cap (12) */
     int32_t reserved;
-    int64_t max_steps;           /* step attempts per leg before KETE_BODY_STEP_CAP */
+    int64_t max_steps;           /* step attempts per leg before KETE_BODY_STEP_CAP (a leg
+                                  * from stop to stop; the lanes' steps, rounded down to
+                                  * the step grid's, are a few more than the warps') */
     /* Per-body non-gravitational terms: device array of one kete_nongrav per
      * body of the call, indexed like its states (8-byte aligned), or NULL
      * (default).  Read by kete_propagate, kete_propagate_stops,
@@ -148,7 +150,10 @@ typedef struct kete_survey_opts {
     double batch_span;           /* a batch holds epochs t with t - t_first < span (3 days) */
     double twobody_max;          /* longest two-body interval (1.5 days); 0 = n-body to every epoch */
     double cell_deg;             /* sky-cell size for candidate search; 0 = automatic */
-    double mem_budget_gb;        /* device scratch budget for batch states (0 = 8 GB) */
+    double mem_budget_gb;        /* device scratch budget for batch states (0 = 8 GB);
+                                  * steps end where a chunk of batches ends, so another
+                                  * budget gives another step sequence (differences at
+                                  * the truncation level) */
 } kete_survey_opts;
 
 /* One body inside one polygon.  Hits come back sorted by (frame, body). */
@@ -365,10 +370,13 @@ int kete_get_stats(const kete_ctx *ctx, kete_stats *out);
  * stop reached (the three values of split_lanes act alike).  Without an
  * explicit budget a call of few bodies takes one warp per body throughout; in
  * that form every term is FP64 in both precisions.
- * Which bodies are set aside depends on each body
+ * In a given call which bodies are set aside depends on each body
  * alone, so the static and work-stealing schedules still agree bit for bit;
  * the two forms differ in the order of their sums and corrector sweeps
- * (differences at the truncation level, ~1e-13 AU over a year).  cost_order != 0: lanes take the bodies
+ * (differences at the truncation level, ~1e-13 AU over a year).  The form and
+ * the automatic budget follow the number of bodies and the span, and the step
+ * grid starts at the first body's epoch: a part of a population propagated by
+ * itself agrees with the whole at that level, not bit for bit.  cost_order != 0: lanes take the bodies
  * most expensive first (cost estimated from each body's heliocentric conic:
  * steps ~ integral dt / r^1.5), so a warp holds bodies of similar cost; this
  * changes only the schedule, not any result.  Default: work stealing, 128, no
@@ -412,9 +420,13 @@ typedef struct kete_obs {
  * projection (differentiation of the path of Sec. 2 / App. A).
  * Forward model of body i: its observations obs[i][0..m) (device, [n][m],
  * sorted by epoch) are batched by the <= batch_span rule (opt, Sec. 2); the
- * n-body chain visits the batch midpoints and the checkpoint grid
- * epochs[i] + ckpt_days * k (k >= 1, before the last midpoint); two-body +
- * light time + RA/Dec give each observation's prediction.
+ * n-body chain visits the batch midpoints; two-body +
+ * light time + RA/Dec give each observation's prediction.  With fm->nongrav,
+ * max_iter < 8, the Sun inactive or more than 12 active masses (3 besides the
+ * Sun with GR or J2 terms) every step ends at the midpoints and at the checkpoint
+ * grid epochs[i] + ckpt_days * k (k >= 1, before the last midpoint);
+ * otherwise steps pass them, and the grid counts toward KETE_ADJ_MAX_STEPS (a
+ * step that passes stops as one for each) and cuts max_steps' legs.
  *   loss[i] = sum_j (wrap(RA_j - RA_obs_j) cos Dec_obs_j)^2 + (Dec_j - Dec_obs_j)^2
  * (device, [n]); grad (device, [6][n], may be NULL) = d loss[i] / d(x0, v0)
  * from the adjoint equations integrated backward over every stored forward
