@@ -71,7 +71,8 @@ __device__ __forceinline__ double ckpts_before(double inv_ckpt, double epoch0, d
 // years of 8-day legs, 183 steps there, came to 281.)
 __device__ __forceinline__ int steps_with_stops(double ckpts, int midpoints)
 {
-    return max(1, (int)fmin(ckpts, 1e6) + midpoints);
+    const int stops = (int)fmin(ckpts, 1e6) + midpoints;
+    return stops > 1 ? stops : 1;
 }
 
 // observations in use: those before the first non-finite epoch
